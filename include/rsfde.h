@@ -260,7 +260,9 @@ int rsfde_apply_M(rsfde_ctx* ctx, const double* z, double* w);
  * resid_prec, RSFDE_FP64 or RSFDE_EXACT (RSFDE_DF32: RSFDE_EINVAL).  x, b, r
  * device N doubles (r distinct from x and b). */
 int rsfde_residual(rsfde_ctx* ctx, const double* x, const double* b, double* r);
-/* Eq. 4.6: z = P-hat^-1 v in the context's preconditioner precision (result in FP64). */
+/* Eq. 4.6: z = P-hat^-1 v in the context's preconditioner precision (result in FP64).
+ * (FP64, and rsfde_dst2: if a device-side wait gives up, the values it left
+ * incomplete are NaN, and the next solve or step returns RSFDE_ETIMEOUT.) */
 int rsfde_apply_precond(rsfde_ctx* ctx, const double* v, double* z);
 /* Section 4.1: out = (S_{n2} (x) S_{n1}) v, the orthonormal 2D sine transform, FP64. */
 int rsfde_dst2(rsfde_ctx* ctx, const double* v, double* out);
@@ -314,9 +316,11 @@ int rsfde_dst2_noalloc(int32_t n1, int32_t n2, const double* v, double* out, voi
 #define RSFDE_K_UPDATE 6        /* Arnoldi update, norm and Givens step */
 #define RSFDE_K_XUPDATE 7       /* solution update x += Z y */
 #define RSFDE_K_OTHER 8         /* right side, norms, scalar kernels */
-#define RSFDE_K_DST_GEMM 9      /* preconditioner as tensor-core GEMMs (split-BF16 or BF16): the four
-                                   GEMMs and, when the previous Gram-Schmidt update did not write the
-                                   first operand, the split */
+#define RSFDE_K_DST_GEMM 9      /* preconditioner (and rsfde_dst2) as tensor-core GEMMs: split-BF16 or
+                                   BF16 (the four GEMMs and, when the previous Gram-Schmidt update did
+                                   not write the first operand, the split), or FP64 by digit products
+                                   (four splits and four products; sides up to 2048, not in paper mode:
+                                   there, and beyond, FP64 runs as FFTs) */
 #define RSFDE_K_RESID_ROWS 10   /* row pass of M x in the true residual (Eq. 2.15) */
 #define RSFDE_K_RESID_COLS 11   /* column pass of the true residual b - M x and its norm */
 #define RSFDE_K_SOLVE_Y 12      /* back substitution of the Givens-rotated least squares */
@@ -350,7 +354,7 @@ const char* rsfde_kernel_class_name(int k);
 int rsfde_autotune(rsfde_ctx* ctx, int32_t reps, int32_t* chosen);
 int rsfde_batch_autotune(rsfde_batch* b, int32_t reps);
 
-/* Failure detection.  Every wait of the tensor-core preconditioner's
+/* Failure detection.  Every wait of the tensor-core preconditioners'
  * pipeline (a TMA copy landing in a ring slot, a slot freed by the MMAs) is
  * bounded; a wait that runs out makes that launch give up and the call
  * return RSFDE_ETIMEOUT, after every copy and MMA the launch had issued has

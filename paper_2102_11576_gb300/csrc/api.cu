@@ -243,7 +243,8 @@ struct rsfde_ctx {
   SolverState* st_host = nullptr;  // pinned
   int64_t launches = 0;
   Bf16Plan* bf16 = nullptr;  // tensor-core preconditioner, made when first needed
-  long long wait_cycles = 0;  // its pipeline wait bound (0: the default)
+  DigitPlan* digit = nullptr;  // FP64 preconditioner as digit products (nullptr: FP64 FFTs)
+  long long wait_cycles = 0;  // their pipeline wait bound (0: the default)
   // one FGMRES cycle captured as the body of a device-side WHILE loop
   cudaStream_t cap_stream = nullptr;  // private stream used only for capture
   cudaGraph_t graph = nullptr;
@@ -347,6 +348,7 @@ int build_tables(rsfde_ctx* c) {
   if ((e = c->ydf.upload(c->hy_axis, c->stream)) != cudaSuccess) return cuda_fail(e);
   if ((e = c->xex.upload(c->hx_axis, c->stream)) != cudaSuccess) return cuda_fail(e);
   if ((e = c->yex.upload(c->hy_axis, c->stream)) != cudaSuccess) return cuda_fail(e);
+  if (c->digit) digit_plan_params(c->digit, c->x64.tab.lam, c->y64.tab.lam, c->pen, c->stream);
   return RSFDE_OK;
 }
 
@@ -373,6 +375,7 @@ void free_ctx(rsfde_ctx* c) {
   if (c->graph) cudaGraphDestroy(c->graph);
   if (c->cap_stream) cudaStreamDestroy(c->cap_stream);
   bf16_plan_destroy(c->bf16);
+  digit_plan_destroy(c->digit);
   delete c;
 }
 
@@ -399,6 +402,36 @@ int ensure_bf16(rsfde_ctx* c) {
   const int rc = bf16_plan_create(&c->bf16, c->n1, c->n2, nt, c->x32.tab.lam, c->y32.tab.lam, c->phi, c->stream);
   if (rc == RSFDE_OK) bf16_plan_set_wait(c->bf16, c->wait_cycles);
   return rc;
+}
+
+// The FP64 preconditioner runs as digit products on the tensor cores
+// (digit.cuh) where their exactness bound allows the sides (n <= 2048), else --
+// and where the plan's memory cannot be had -- by FP64 FFTs.  One application,
+// digits against FFTs: 64 x 64 49 us / 100 us, 512 x 512 112 / 370, 1023 x 641
+// 0.24 ms / 1.79, 2048 x 2048 1.31 ms / 7.68.  Paper mode keeps the FFTs: its stop test ||P^-1 (b - M x)|| at 1e-8
+// is near what FP64 resolves of the penalty rows (dt/eta x cancels in b - M x),
+// so its iteration counts, which reproduce the paper's tables, depend on the rounding.
+bool left_variant(const rsfde_ctx* c) { return c->opts.variant == RSFDE_GMRES_LEFT; }
+int ensure_digits(rsfde_ctx* c) {
+  if (c->digit || c->opts.precond_prec != RSFDE_FP64 || !c->opts.use_precond || left_variant(c) ||
+      !digit_sizes_ok(c->n1, c->n2))
+    return RSFDE_OK;
+  if (digit_plan_create(&c->digit, c->n1, c->n2, c->stream) != RSFDE_OK) return RSFDE_OK;
+  digit_plan_params(c->digit, c->x64.tab.lam, c->y64.tab.lam, c->pen, c->stream);
+  digit_plan_set_wait(c->digit, c->wait_cycles);
+  return RSFDE_OK;
+}
+bool digit_precond_on(const rsfde_ctx* c) {
+  return c->digit && c->opts.precond_prec == RSFDE_FP64 && !left_variant(c);
+}
+
+// z = P-hat^-1 (scale * v) by digit products (eight launches).
+template <typename Tin>
+void enqueue_precond_digit(rsfde_ctx* c, const Tin* v, const double* vscale, double* z, const int* gate) {
+  ProfScope ps(c, RSFDE_K_DST_GEMM);
+  c->launches += 7;
+  digit_precond<Tin>(c->digit, v, vscale, z, c->phi, static_cast<double*>(c->T1), static_cast<double*>(c->T2a),
+                     static_cast<double*>(c->T2b), gate, c->stream);
 }
 
 // The tensor-core preconditioner z = P-hat^-1 (scale * v) (five launches).
@@ -435,8 +468,6 @@ void enqueue_apply_M(rsfde_ctx* c, const Tz* z, double* w, const int* gate) {
   else enqueue_apply_M_t<double, Tz, double>(c, z, w, gate, c->x64.tab, c->y64.tab);
 }
 
-bool left_variant(const rsfde_ctx* c) { return c->opts.variant == RSFDE_GMRES_LEFT; }
-
 // The right-preconditioned FGMRES keeps its Krylov basis, and runs its
 // Gram-Schmidt, in basis_prec: FP64 (FP64 arithmetic, whatever the operator's
 // arithmetic), or -- with an operator of the same precision, whose output is
@@ -462,6 +493,7 @@ void enqueue_precond_bf16(rsfde_ctx* c, const Tin* v, const double* vscale, Tz* 
 void enqueue_precond64(rsfde_ctx* c, const double* v, const double* vscale, double* z, const int* gate) {
   if (bf16_precond_on(c)) enqueue_precond_bf16<double, double>(c, v, vscale, z, gate);
   else if (fp32_precond(c)) enqueue_precond_t<float, double, double>(c, v, vscale, z, gate, c->x32.tab, c->y32.tab);
+  else if (digit_precond_on(c)) enqueue_precond_digit<double>(c, v, vscale, z, gate);
   else enqueue_precond_t<double, double, double>(c, v, vscale, z, gate, c->x64.tab, c->y64.tab);
 }
 
@@ -631,7 +663,9 @@ void enqueue_cycle_t(rsfde_ctx* c) {
         enqueue_precond_bf16<Tz, Tv>(c, vj, &c->st->s[j], zj, gi, fused && j > 0);
       else if (fp32_precond(c))
         enqueue_precond_t<float, Tz, Tv>(c, vj, &c->st->s[j], zj, gi, c->x32.tab, c->y32.tab);
-      else
+      else if (digit_precond_on(c)) {
+        if constexpr (std::is_same<Tz, double>::value) enqueue_precond_digit<Tv>(c, vj, &c->st->s[j], zj, gi);
+      } else
         enqueue_precond_t<double, Tz, Tv>(c, vj, &c->st->s[j], zj, gi, c->x64.tab, c->y64.tab);
     } else {
       ProfScope ps(c, RSFDE_K_OTHER);
@@ -843,6 +877,7 @@ int run_solver(rsfde_ctx* c, rsfde_stats* stats) {
   const SolverState& h = *c->st_host;
   if (c->opts.use_graph && !c->prof_on) c->launches += (int64_t)h.body_runs * c->launches_per_body;
   if (c->bf16 && bf16_precond_on(c) && (rc = bf16_plan_error(c->bf16, c->stream))) return rc;
+  if (digit_precond_on(c) && (rc = digit_plan_error(c->digit, c->stream))) return rc;
   if (stats) {
     stats->iters = h.iters;
     stats->restarts = h.cycles > 0 ? h.cycles - 1 : 0;
@@ -990,7 +1025,8 @@ int autotune_ctx(rsfde_ctx* c, int reps, int32_t* chosen_out) {
     tune_residual<df>(c, reps, c->xdf.tab, c->ydf.tab, unused);
   }
   if (c->opts.precond_prec == RSFDE_FP32) tune_precond<float>(c, reps, c->x32.tab, c->y32.tab, chosen);
-  else if (c->opts.precond_prec == RSFDE_FP64) tune_precond<double>(c, reps, c->x64.tab, c->y64.tab, chosen);
+  else if (c->opts.precond_prec == RSFDE_FP64 && !digit_precond_on(c))
+    tune_precond<double>(c, reps, c->x64.tab, c->y64.tab, chosen);
   int bn[4] = {0, 0, 0, 0};
   int rc = RSFDE_OK;
   if (bf16_precond_on(c) && (rc = ensure_bf16(c)) == RSFDE_OK)
@@ -1661,6 +1697,7 @@ int rsfde_setup(rsfde_ctx** out, const rsfde_grid* g, const uint8_t* mask, doubl
   }
   int rc = build_tables(c);
   if (rc == RSFDE_OK) rc = ensure_bf16(c);
+  if (rc == RSFDE_OK) rc = ensure_digits(c);
   if (rc == RSFDE_OK) rc = check_launch(c);
   if (rc == RSFDE_OK) rc = cuda_fail(cudaStreamSynchronize(c->stream));
   if (rc != RSFDE_OK) {
@@ -1683,7 +1720,8 @@ int rsfde_set_opts(rsfde_ctx* c, const rsfde_opts* o) {
   if (!c || !o || !valid_opts(o) || o->restart > c->m_alloc) return RSFDE_EINVAL;
   c->opts = *o;
   c->stream = static_cast<cudaStream_t>(o->stream);
-  return ensure_bf16(c);
+  const int rc = ensure_bf16(c);
+  return rc != RSFDE_OK ? rc : ensure_digits(c);
 }
 
 int rsfde_set_stream(rsfde_ctx* c, void* stream) {
@@ -1828,6 +1866,7 @@ int rsfde_apply_precond(rsfde_ctx* c, const double* v, double* z) {
     return bf16_plan_error(c->bf16, c->stream);
   }
   if (fp32_precond(c)) enqueue_precond_t<float, double, double>(c, v, nullptr, z, nullptr, c->x32.tab, c->y32.tab);
+  else if (digit_precond_on(c)) enqueue_precond_digit<double>(c, v, nullptr, z, nullptr);
   else enqueue_precond_t<double, double, double>(c, v, nullptr, z, nullptr, c->x64.tab, c->y64.tab);
   return check_launch(c);
 }
@@ -1835,6 +1874,12 @@ int rsfde_apply_precond(rsfde_ctx* c, const double* v, double* z) {
 int rsfde_dst2(rsfde_ctx* c, const double* v, double* out) {
   NvtxRange range("rsfde_dst2");
   if (!c || !v || !out) return RSFDE_EINVAL;
+  if (c->digit && !left_variant(c)) {
+    ProfScope ps(c, RSFDE_K_DST_GEMM);
+    c->launches += 3;
+    digit_dst2(c->digit, v, out, static_cast<double*>(c->T1), c->stream);
+    return check_launch(c);
+  }
   {
     ProfScope ps(c, RSFDE_K_DST_ROWS);
     launch_dst_rows<double, double, double>(v, nullptr, c->tmpx, c->n1, c->n2, c->x64.tab, nullptr, c->stream);
@@ -1871,6 +1916,7 @@ int rsfde_set_wait_cycles(rsfde_ctx* c, int64_t cycles) {
   if (!c || cycles < 0) return RSFDE_EINVAL;
   c->wait_cycles = cycles;
   bf16_plan_set_wait(c->bf16, cycles);
+  digit_plan_set_wait(c->digit, cycles);
   return RSFDE_OK;
 }
 

@@ -1,5 +1,6 @@
 // internal.h -- declarations shared by the library's translation units.
 #pragma once
+#include <cuda.h>
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
 #include <stdint.h>
@@ -164,6 +165,12 @@ struct Bf16Out {
   int n1, ld, hk;
 };
 
+// cuTensorMapEncodeTiled through the runtime's entry-point lookup (dst_gemm.cu); nullptr if missing
+typedef CUresult (*EncodeTiledFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*,
+                                  const cuuint64_t*, const cuuint32_t*, const cuuint32_t*, CUtensorMapInterleave,
+                                  CUtensorMapSwizzle, CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
+EncodeTiledFn encode_fn();
+
 // ---- split-BF16 tensor-core preconditioner (dst_gemm.cu) --------------------
 struct Bf16Plan;
 // nt: BF16 products per GEMM, 3 (split BF16) or 1 (plain BF16)
@@ -187,6 +194,22 @@ int bf16_plan_autotune(Bf16Plan* p, const double* v, float* z, const uint8_t* ph
 // The Bf16Out target of the plan's first operand, if the plan can take it
 // (symmetric layout, n1 a multiple of vec); returns false otherwise.
 bool bf16_plan_a0(const Bf16Plan* p, int vec, Bf16Out* out);
+
+// ---- FP64 sine transforms as digit products on the tensor cores (digit.cu) ---
+struct DigitPlan;
+bool digit_sizes_ok(int n1, int n2);  // the sides the digit products take (both <= 2048)
+int digit_plan_create(DigitPlan** out, int n1, int n2, cudaStream_t s);
+void digit_plan_destroy(DigitPlan* p);
+// the tabulated reciprocals of the tau divides (enqueued on s)
+void digit_plan_params(DigitPlan* p, const double* lamx, const double* lamy, double pen, cudaStream_t s);
+int digit_plan_error(DigitPlan* p, cudaStream_t s);  // reads and clears the give-up flag
+void digit_plan_set_wait(DigitPlan* p, long long cycles);  // <= 0: the default bound
+// z = P-hat^-1 (scale v) in eight launches; t, wa, wb: N doubles of scratch each
+template <typename Tin>
+void digit_precond(DigitPlan* p, const Tin* v, const double* vscale, double* z, const uint8_t* phi, double* t,
+                   double* wa, double* wb, const int* gate, cudaStream_t s);
+// out = (S_{n2} (x) S_{n1}) v in four launches; t: N doubles of scratch
+void digit_dst2(DigitPlan* p, const double* v, double* out, double* t, cudaStream_t s);
 
 // ---- batched instances: one launch per phase over every instance -------------
 // One instance of a batch as the multi-instance kernels see it (an array of
