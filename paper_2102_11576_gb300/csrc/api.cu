@@ -244,6 +244,7 @@ struct rsfde_ctx {
   int64_t launches = 0;
   Bf16Plan* bf16 = nullptr;  // tensor-core preconditioner, made when first needed
   DigitPlan* digit = nullptr;  // FP64 preconditioner as digit products (nullptr: FP64 FFTs)
+  DigitOperator* dop = nullptr;  // FP64 operator likewise
   long long wait_cycles = 0;  // their pipeline wait bound (0: the default)
   // one FGMRES cycle captured as the body of a device-side WHILE loop
   cudaStream_t cap_stream = nullptr;  // private stream used only for capture
@@ -349,6 +350,11 @@ int build_tables(rsfde_ctx* c) {
   if ((e = c->xex.upload(c->hx_axis, c->stream)) != cudaSuccess) return cuda_fail(e);
   if ((e = c->yex.upload(c->hy_axis, c->stream)) != cudaSuccess) return cuda_fail(e);
   if (c->digit) digit_plan_params(c->digit, c->x64.tab.lam, c->y64.tab.lam, c->pen, c->stream);
+  if (c->dop && !digit_operator_params(c->dop, c->hx_axis.t, c->hy_axis.t, c->stream)) {
+    digit_operator_destroy(c->dop);  // the FFTs take over
+    c->dop = nullptr;
+    c->graph_key = -1;
+  }
   return RSFDE_OK;
 }
 
@@ -376,6 +382,7 @@ void free_ctx(rsfde_ctx* c) {
   if (c->cap_stream) cudaStreamDestroy(c->cap_stream);
   bf16_plan_destroy(c->bf16);
   digit_plan_destroy(c->digit);
+  digit_operator_destroy(c->dop);
   delete c;
 }
 
@@ -412,7 +419,27 @@ int ensure_bf16(rsfde_ctx* c) {
 // is near what FP64 resolves of the penalty rows (dt/eta x cancels in b - M x),
 // so its iteration counts, which reproduce the paper's tables, depend on the rounding.
 bool left_variant(const rsfde_ctx* c) { return c->opts.variant == RSFDE_GMRES_LEFT; }
+// The FP64 operator on the Arnoldi vectors runs as digit products by the same
+// rule.  M z, digits against FFTs: 64 x 64 28 us / 56, 300 x 1500 89 / 218, 512 x
+// 512 55 / 93, 2048 x 2048 0.51 ms / 1.53.
+int ensure_digit_operator(rsfde_ctx* c) {
+  if (c->dop || c->opts.matvec_prec != RSFDE_FP64 || left_variant(c) || !digit_sizes_ok(c->n1, c->n2)) return RSFDE_OK;
+  if (digit_operator_create(&c->dop, c->n1, c->n2, c->stream) != RSFDE_OK) return RSFDE_OK;
+  if (!digit_operator_params(c->dop, c->hx_axis.t, c->hy_axis.t, c->stream)) {
+    cudaGetLastError();
+    digit_operator_destroy(c->dop);
+    c->dop = nullptr;
+    return RSFDE_OK;
+  }
+  digit_operator_set_wait(c->dop, c->wait_cycles);
+  return RSFDE_OK;
+}
+bool digit_operator_on(const rsfde_ctx* c) {
+  return c->dop && c->opts.matvec_prec == RSFDE_FP64 && !left_variant(c);
+}
 int ensure_digits(rsfde_ctx* c) {
+  const int rc = ensure_digit_operator(c);
+  if (rc != RSFDE_OK) return rc;
   if (c->digit || c->opts.precond_prec != RSFDE_FP64 || !c->opts.use_precond || left_variant(c) ||
       !digit_sizes_ok(c->n1, c->n2))
     return RSFDE_OK;
@@ -465,7 +492,11 @@ void enqueue_apply_M(rsfde_ctx* c, const Tz* z, double* w, const int* gate) {
   if (c->opts.matvec_prec == RSFDE_DF32) enqueue_apply_M_t<df, Tz, double>(c, z, w, gate, c->xdf.tab, c->ydf.tab);
   else if (c->opts.matvec_prec == RSFDE_FP32)
     enqueue_apply_M_t<float, Tz, double>(c, z, w, gate, c->x32.tab, c->y32.tab);
-  else enqueue_apply_M_t<double, Tz, double>(c, z, w, gate, c->x64.tab, c->y64.tab);
+  else if (digit_operator_on(c)) {
+    ProfScope ps(c, RSFDE_K_TOEPLITZ_COLS);
+    c->launches += 2;
+    digit_apply_M<Tz>(c->dop, z, w, c->phi, c->pen, c->tmpx, gate, c->stream);
+  } else enqueue_apply_M_t<double, Tz, double>(c, z, w, gate, c->x64.tab, c->y64.tab);
 }
 
 // The right-preconditioned FGMRES keeps its Krylov basis, and runs its
@@ -877,7 +908,9 @@ int run_solver(rsfde_ctx* c, rsfde_stats* stats) {
   const SolverState& h = *c->st_host;
   if (c->opts.use_graph && !c->prof_on) c->launches += (int64_t)h.body_runs * c->launches_per_body;
   if (c->bf16 && bf16_precond_on(c) && (rc = bf16_plan_error(c->bf16, c->stream))) return rc;
-  if (digit_precond_on(c) && (rc = digit_plan_error(c->digit, c->stream))) return rc;
+  const int e1 = digit_precond_on(c) ? digit_plan_error(c->digit, c->stream) : RSFDE_OK;
+  const int e2 = digit_operator_on(c) ? digit_operator_error(c->dop, c->stream) : RSFDE_OK;
+  if (e1 || e2) return e1 ? e1 : e2;
   if (stats) {
     stats->iters = h.iters;
     stats->restarts = h.cycles > 0 ? h.cycles - 1 : 0;
@@ -1015,7 +1048,7 @@ int autotune_ctx(rsfde_ctx* c, int reps, int32_t* chosen_out) {
   } else if (c->opts.matvec_prec == RSFDE_FP32) {
     if (b64) tune_operator<float, double>(c, reps, c->x32.tab, c->y32.tab, chosen);
     else tune_operator<float, float>(c, reps, c->x32.tab, c->y32.tab, chosen);
-  } else {
+  } else if (!digit_operator_on(c)) {
     tune_operator<double, double>(c, reps, c->x64.tab, c->y64.tab, chosen);
   }
   // the double-FP32 true residual runs the same transform families in 8-byte
@@ -1917,6 +1950,7 @@ int rsfde_set_wait_cycles(rsfde_ctx* c, int64_t cycles) {
   c->wait_cycles = cycles;
   bf16_plan_set_wait(c->bf16, cycles);
   digit_plan_set_wait(c->digit, cycles);
+  digit_operator_set_wait(c->dop, cycles);
   return RSFDE_OK;
 }
 

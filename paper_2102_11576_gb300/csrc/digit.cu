@@ -10,6 +10,13 @@
 //   2. T^T             -> digits,  W1, W2 from T^T S_y          (each n2 x n1)
 //   3. [W1; W2]        -> digits,  Y^T  = ([W1; W2] S_x)^T      (two n1 x n2)
 //   4. Y^T             -> digits,  z = S_y Y_c where the mask selects channel c
+// The operator M z (Eq. 2.14-2.17) is two more such products, with the symmetric
+// Toeplitz matrices in place of S: they are centrosymmetric too (T[n-1-i][n-1-j]
+// = T[i][j]), so with z+_j = z_j + z_{n-1-j} and z-_j = z_j - z_{n-1-j}
+//     (T z)_i, (T z)_{n-1-i} = sum_j U_ij z+_j +- sum_j V_ij z-_j,
+//     U_ij, V_ij = (T_ij +- T_{i,n-1-j}) / 2,   i, j < (n+1)/2:
+// the layout of the symmetric sine product, half the work of the full one.
+//
 // A product's epilogue also finds the largest exponent of every row of its
 // output, so the next split is one elementwise pass.
 #include <cmath>
@@ -60,6 +67,19 @@ __device__ __forceinline__ void store_digits(const long long* q, __nv_bfloat16* 
     *reinterpret_cast<uint2*>(p) = make_uint2(dg_pack(v[0], v[2]), dg_pack(v[4], v[6]));
     *reinterpret_cast<uint2*>(p + hk) = make_uint2(dg_pack(v[1], v[3]), dg_pack(v[5], v[7]));
   }
+}
+
+// The digits of four quantised values p (to columns 4c .. 4c + 3 of the first
+// half) and m (of the second half).
+__device__ __forceinline__ void store_digits4(const long long* p, const long long* m, __nv_bfloat16* row, size_t plane,
+                                              int hk, int c) {
+  long long q[8];
+#pragma unroll
+  for (int k = 0; k < 4; ++k) {
+    q[2 * k] = p[k];
+    q[2 * k + 1] = m[k];
+  }
+  store_digits(q, row, plane, hk, c);
 }
 
 // The first operand: rows y of scale * v (one block per row, one group of
@@ -193,6 +213,152 @@ __global__ void __launch_bounds__(256)
   if (threadIdx.x < 2) atomicMax(rowsum, half[threadIdx.x]);
 }
 
+// Both operands of the operator from z, in one launch, and the part of M z that
+// is not left to the products.  The first `rblocks` blocks take the rows (one or
+// more warps each): row y folded (z+, z-) to digits dr, its exponent to er[y], and
+//     pre = (1 - t0x - t0y) z - t1x (z_left + z_right) - t1y (z_below + z_above),
+// the identity and the three middle diagonals of both Toeplitz matrices in FP64.  The others take CPB columns each, held in shared memory
+// (read once, for the largest entries and for the digits): digits dc (rows x),
+// exponents ec[x].
+//
+// The middle diagonals stay out of the digits because they are 48 to 130 times
+// the next ones: the products' absolute error is set by the largest coefficient
+// and would be 1e-15 to 5e-15 of M z (an FP64 FFT: 2e-16 to 3e-16), and is 48
+// times smaller without them; measured over 1 x 1 .. 2048 x 64, M z is then
+// within 1.6e-16 (2-norm) of the extended-precision product, the FFTs 3.2e-16.
+template <typename Tin, int CPB>
+__global__ void __launch_bounds__(256)
+    digit_fold_kernel(const Tin* __restrict__ z, int n1, int n2, int rblocks, const double* __restrict__ near, double* __restrict__ pre,
+                      __nv_bfloat16* __restrict__ dr, size_t pr, int h1, int* __restrict__ er,
+                      __nv_bfloat16* __restrict__ dc, size_t pc, int h2, int* __restrict__ ec, int* err,
+                      const int* gate) {
+  pdl_wait();
+  pdl_trigger();
+  if (gate && *(volatile const int*)gate == 0) return;
+  __shared__ uint32_t wmax[8][CPB];
+  extern __shared__ __align__(16) double fold_sm[];
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  if (blockIdx.x == 0 && tid == 0) *err = 0;
+  if ((int)blockIdx.x < rblocks) {
+    const int wpr = (h1 / 4 + 31) / 32, rpb = 8 / wpr;  // warps per row (at most 8), rows per block
+    const int y = blockIdx.x * rpb + warp / wpr, c = (warp % wpr) * 32 + lane, half = (n1 + 1) / 2;
+    const bool row = warp / wpr < rpb && y < n2;
+    double a[4], b[4];  // z_j and its mirror
+    uint32_t e = 0;
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      const int j = 4 * c + k;
+      const bool in = row && j < half;
+      a[k] = in ? cvt<double>(z[(size_t)y * n1 + j]) : 0.0;
+      b[k] = in ? cvt<double>(z[(size_t)y * n1 + n1 - 1 - j]) : 0.0;
+      e = max(e, max(dg_exponent(a[k]), dg_exponent(b[k])));
+    }
+    e = __reduce_max_sync(0xffffffffu, e);
+    if (lane == 0) wmax[warp][0] = e;
+    __syncthreads();
+    if (!row) return;
+    for (int w = 0; w < wpr; ++w) e = max(e, wmax[warp / wpr * wpr + w][0]);
+    if (c == 0) er[y] = e == 2047 ? kDgNan : (e ? (int)e : 1) + 1;
+    if (4 * c >= h1) return;
+    const double c0 = __ldg(near), t1x = __ldg(near + 1), t1y = __ldg(near + 2);
+    long long p[4], m[4];
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      const int j = 4 * c + k, E = (e ? (int)e : 1) + 1;
+      const bool mid = 2 * j + 1 == n1;
+      const long long qa = e == 2047 ? 0 : dg_quantize(a[k], E);
+      const long long qb = (e == 2047 || mid) ? 0 : dg_quantize(b[k], E);  // the middle once
+      p[k] = qa + qb;
+      m[k] = mid ? 0 : qa - qb;
+      if (j < half) {
+#pragma unroll
+        for (int mir = 0; mir < 2; ++mir) {
+          if (mir && mid) break;
+          const int x = mir ? n1 - 1 - j : j;
+          const size_t o = (size_t)y * n1 + x;
+          const double sx = (x > 0 ? cvt<double>(z[o - 1]) : 0.0) + (x + 1 < n1 ? cvt<double>(z[o + 1]) : 0.0);
+          const double sy = (y > 0 ? cvt<double>(z[o - n1]) : 0.0) + (y + 1 < n2 ? cvt<double>(z[o + n1]) : 0.0);
+          const double v = __fma_rn(-t1x, sx, c0 * (mir ? b[k] : a[k]));
+          pre[o] = __fma_rn(-t1y, sy, v);
+        }
+      }
+    }
+    store_digits4(p, m, dr + (size_t)y * 2 * h1, pr, h1, c);
+    return;
+  }
+  const int x0 = (blockIdx.x - rblocks) * CPB, ncol = min(CPB, n1 - x0), half = (n2 + 1) / 2;
+  const int ld = n2 + 1;
+  uint32_t e[CPB] = {0};
+  for (int y = tid; y < n2; y += blockDim.x) {
+#pragma unroll
+    for (int c = 0; c < CPB; ++c) {
+      const double v = c < ncol ? cvt<double>(z[(size_t)y * n1 + x0 + c]) : 0.0;
+      fold_sm[c * ld + y] = v;
+      e[c] = max(e[c], dg_exponent(v));
+    }
+  }
+#pragma unroll
+  for (int c = 0; c < CPB; ++c) {
+    const uint32_t w = __reduce_max_sync(0xffffffffu, e[c]);
+    if (lane == 0) wmax[warp][c] = w;
+  }
+  __syncthreads();
+  if (tid < ncol) {
+    uint32_t w = 0;
+    for (int k = 0; k < 8; ++k) w = max(w, wmax[k][tid]);
+    ec[x0 + tid] = w == 2047 ? kDgNan : (w ? (int)w : 1) + 1;
+  }
+  const int gpc = h2 >> 2;  // groups of four per column
+  for (int t = tid; t < ncol * gpc; t += blockDim.x) {
+    const int c = t / gpc, g = t - c * gpc;
+    uint32_t w = 0;
+#pragma unroll
+    for (int k = 0; k < 8; ++k) w = max(w, wmax[k][c]);
+    const int E = (w ? (int)w : 1) + 1;
+    long long p[4], m[4];
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      const int j = 4 * g + k;
+      const bool in = j < half && w != 2047, mid = 2 * j + 1 == n2;
+      const long long qa = in ? dg_quantize(fold_sm[c * ld + j], E) : 0;
+      const long long qb = (in && !mid) ? dg_quantize(fold_sm[c * ld + n2 - 1 - j], E) : 0;
+      p[k] = qa + qb;
+      m[k] = mid ? 0 : qa - qb;
+    }
+    store_digits4(p, m, dc + (size_t)(x0 + c) * 2 * h2, pc, h2, g);
+  }
+}
+
+// The digits of [2U | 2V] from tq[k] = round(2^sh t_k); one block per row i < (n + 1) / 2.
+__global__ void __launch_bounds__(256)
+    digit_toeplitz_kernel(const long long* __restrict__ tq, int n, __nv_bfloat16* __restrict__ d, size_t plane, int hk,
+                          int* rowsum) {
+  const int i = blockIdx.x, half = (n + 1) / 2;
+  __shared__ int hsum[2];
+  if (threadIdx.x < 2) hsum[threadIdx.x] = 0;
+  __syncthreads();
+  int sum[2] = {0, 0};
+  for (int c = threadIdx.x; 4 * c < hk; c += blockDim.x) {
+    long long u[4], v[4];
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      const int j = 4 * c + k;
+      const long long a = j < half ? tq[abs(i - j)] : 0, b = j < half ? tq[abs(i - (n - 1 - j))] : 0;
+      u[k] = a + b;
+      v[k] = a - b;
+      for (int g = 0; g < kDgDigits; ++g) {
+        sum[0] += abs((int)dg_digit((unsigned long long)(u[k] + kDgBias), g) - 64);
+        sum[1] += abs((int)dg_digit((unsigned long long)(v[k] + kDgBias), g) - 64);
+      }
+    }
+    store_digits4(u, v, d + (size_t)i * 2 * hk, plane, hk, c);
+  }
+  atomicAdd(&hsum[0], sum[0]);
+  atomicAdd(&hsum[1], sum[1]);
+  __syncthreads();
+  if (threadIdx.x < 2) atomicMax(rowsum, hsum[threadIdx.x]);
+}
+
 // 1 / (1 - lx - ly) and 1 / (1 + dt/eta - lx - ly) at [y * n1 + x]
 __global__ void __launch_bounds__(kBlock)
     digit_reciprocals_kernel(const double* __restrict__ lx, const double* __restrict__ ly, double pen, int n1, int n2,
@@ -318,13 +484,14 @@ void digit_plan_params(DigitPlan* p, const double* lamx, const double* lamy, dou
   digit_reciprocals_kernel<<<vec_grid(N), kBlock, 0, s>>>(lamx, lamy, pen, p->n1, p->n2, p->inv, p->inv + N);
 }
 
-int digit_plan_error(DigitPlan* p, cudaStream_t s) {
+static int digit_error(int* err, cudaStream_t s) {
   int h = 0;
-  if (cudaMemcpyAsync(&h, p->err + 1, sizeof(int), cudaMemcpyDeviceToHost, s) != cudaSuccess) return RSFDE_ECUDA;
+  if (cudaMemcpyAsync(&h, err + 1, sizeof(int), cudaMemcpyDeviceToHost, s) != cudaSuccess) return RSFDE_ECUDA;
   if (cudaStreamSynchronize(s) != cudaSuccess) return RSFDE_ECUDA;
-  if (h && cudaMemsetAsync(p->err, 0, 2 * sizeof(int), s) != cudaSuccess) return RSFDE_ECUDA;
+  if (h && cudaMemsetAsync(err, 0, 2 * sizeof(int), s) != cudaSuccess) return RSFDE_ECUDA;
   return h ? RSFDE_ETIMEOUT : RSFDE_OK;
 }
+int digit_plan_error(DigitPlan* p, cudaStream_t s) { return digit_error(p->err, s); }
 
 void digit_plan_set_wait(DigitPlan* p, long long cycles) {
   if (p) p->wait_cycles = cycles > 0 ? cycles : kWaitCycles;
@@ -372,11 +539,11 @@ static void launch_digit_bn(const DigitMat& A, const DigitMat& S, const DigitEpi
              S.map[BN == 64 ? 0 : BN == 32 ? 1 : 2], ep, err, gate);
 }
 // A S for a transform of length n
-template <int EPI>
-static void launch_digit(const DigitPlan* p, const DigitMat& A, const DigitMat& S, int n, int kexp,
+template <int EPI, typename Plan>
+static void launch_digit(const Plan* p, const DigitMat& A, const DigitMat& S, int n, int kexp,
                          DigitEpiParams ep, const int* gate, cudaStream_t s) {
-  ep.M = A.rows;
-  ep.N = (n + 1) / 2;
+  ep.M = A.rows;  // (DG_ROWS: A the matrix, S the operand's rows)
+  ep.N = S.rows;
   ep.n_full = n;
   ep.hk = A.hk;
   ep.kexp = kexp;
@@ -456,6 +623,149 @@ void digit_dst2(DigitPlan* p, const double* v, double* out, double* t, cudaStrea
   ep.ldo = p->n1;
   launch_digit<DG_STORE>(p, p->T, p->Sy, p->n2, p->ky, ep, nullptr, s);
 }
+
+// ---- the operator ------------------------------------------------------------
+struct DigitOperator {
+  int n1 = 0, n2 = 0;
+  DigitMat Tx, Ty, R, C;  // [U | V] of each axis; the rows and the columns of z
+  int* exps = nullptr;     // n2 (rows), n1 (columns)
+  int* err = nullptr;
+  // the parameters, on the device (captured launches read them where they are):
+  double* near = nullptr;  // 1 - t0x - t0y, t1x, t1y
+  int* kexp = nullptr;     // the scales of the two products
+  long long* tq = nullptr;
+  void* mem = nullptr;
+  long long wait_cycles = kWaitCycles;
+};
+
+// [2U | 2V] of t without its first two entries; *kexp the scale of a product with it.
+static bool build_toeplitz(DigitOperator* p, DigitMat* T, const std::vector<double>& t, int* kexp, cudaStream_t s) {
+  const int n = (int)t.size();
+  double big = 0.0;
+  for (int k = 2; k < n; ++k) big = std::fmax(big, std::fabs(t[k]));
+  int E = 0;
+  std::frexp(big, &E);  // |t_k| < 2^E
+  std::vector<long long> q(n, 0);
+  for (int extra = 0; extra < 3; ++extra) {
+    const int sh = 54 - (E + extra);  // |2U|, |2V| <= 2^55
+    for (int k = 2; k < n; ++k) q[k] = std::llround(std::ldexp(t[k], sh));
+    int rowsum = 0;
+    if (cudaMemcpyAsync(p->tq, q.data(), n * sizeof(long long), cudaMemcpyHostToDevice, s) != cudaSuccess ||
+        cudaMemsetAsync(p->err + 2, 0, sizeof(int), s) != cudaSuccess)
+      return false;
+    digit_toeplitz_kernel<<<T->rows, 256, 0, s>>>(p->tq, n, T->d, T->plane(), T->hk, p->err + 2);
+    if (cudaMemcpyAsync(&rowsum, p->err + 2, sizeof(int), cudaMemcpyDeviceToHost, s) != cudaSuccess ||
+        cudaStreamSynchronize(s) != cudaSuccess)
+      return false;
+    // z = z_q 2^(E_z - 1077), 2U = U_q 2^-sh, sum z U = W 2^(9 + 49 - 1) 2^(E_z - 1077 - sh)
+    *kexp = 57 - 1077 - sh;
+    if (64LL * rowsum <= (1LL << 24)) return true;
+  }
+  return false;
+}
+
+bool digit_operator_params(DigitOperator* p, const std::vector<double>& tx, const std::vector<double>& ty,
+                           cudaStream_t s) {
+  int k[2];
+  if (!build_toeplitz(p, &p->Tx, tx, &k[0], s) || !build_toeplitz(p, &p->Ty, ty, &k[1], s)) return false;
+  const double near[3] = {1.0 - tx[0] - ty[0], tx.size() > 1 ? tx[1] : 0.0, ty.size() > 1 ? ty[1] : 0.0};
+  return cudaMemcpyAsync(p->near, near, sizeof(near), cudaMemcpyHostToDevice, s) == cudaSuccess &&
+         cudaMemcpyAsync(p->kexp, k, sizeof(k), cudaMemcpyHostToDevice, s) == cudaSuccess &&
+         cudaStreamSynchronize(s) == cudaSuccess;
+}
+
+int digit_operator_create(DigitOperator** out, int n1, int n2, cudaStream_t s) {
+  *out = nullptr;
+  if (!digit_sizes_ok(n1, n2)) return RSFDE_EINVAL;
+  DigitOperator* p = new (std::nothrow) DigitOperator();
+  if (!p) return RSFDE_ENOMEM;
+  p->n1 = n1;
+  p->n2 = n2;
+  const int h1 = pad16((n1 + 1) / 2), h2 = pad16((n2 + 1) / 2);
+  size_t off[5] = {0, 0, 0, 0, 0};
+  DigitMat* mats[4] = {&p->Tx, &p->Ty, &p->R, &p->C};
+  const int rows[4] = {(n1 + 1) / 2, (n2 + 1) / 2, n2, n1}, hk[4] = {h1, h2, h1, h2};
+  for (int k = 0; k < 4; ++k) {
+    mats[k]->rows = rows[k];
+    mats[k]->hk = hk[k];
+    off[k + 1] = off[k] + (mats[k]->plane() * kDgDigits * 2 + 255) / 256 * 256;
+  }
+  const size_t se = ((size_t)(n1 + n2) * sizeof(int) + 255) / 256 * 256;
+  if (cudaMalloc(&p->mem, off[4] + se + 256 + kDgMaxN * sizeof(long long)) != cudaSuccess) {
+    cudaGetLastError();
+    delete p;
+    return RSFDE_ENOMEM;
+  }
+  uint8_t* b = static_cast<uint8_t*>(p->mem);
+  for (int k = 0; k < 4; ++k) mats[k]->d = reinterpret_cast<__nv_bfloat16*>(b + off[k]);
+  p->exps = reinterpret_cast<int*>(b + off[4]);
+  p->err = reinterpret_cast<int*>(b + off[4] + se);
+  p->near = reinterpret_cast<double*>(b + off[4] + se + 64);
+  p->kexp = reinterpret_cast<int*>(b + off[4] + se + 128);
+  p->tq = reinterpret_cast<long long*>(b + off[4] + se + 256);
+  bool good = cudaMemsetAsync(p->err, 0, 256, s) == cudaSuccess;
+  good = good && digit_map(&p->Tx, &p->Tx.map[0], kDgBM, 1) && digit_map(&p->C, &p->C.map[0], kDgBM, 1);
+  for (DigitMat* m : {&p->R, &p->Ty})
+    for (int k = 0; k < 3; ++k) good = good && digit_map(m, &m->map[k], 64 >> k, kDgDigits);
+  if (!good) {
+    cudaGetLastError();
+    digit_operator_destroy(p);
+    return RSFDE_ECUDA;
+  }
+  *out = p;
+  return RSFDE_OK;
+}
+
+void digit_operator_destroy(DigitOperator* p) {
+  if (!p) return;
+  if (p->mem) cudaFree(p->mem);
+  delete p;
+}
+int digit_operator_error(DigitOperator* p, cudaStream_t s) { return digit_error(p->err, s); }
+void digit_operator_set_wait(DigitOperator* p, long long cycles) {
+  if (p) p->wait_cycles = cycles > 0 ? cycles : kWaitCycles;
+}
+
+// Columns per block of the fold: four (32-byte pieces of z's rows, 64 KB at n2 =
+// 2048: three blocks per SM) while that gives every SM a block, else two.
+template <typename Tin, int CPB>
+static void launch_fold(DigitOperator* p, const Tin* z, double* pre, const int* gate, cudaStream_t s) {
+  const int n1 = p->n1, n2 = p->n2, wpr = (p->R.hk / 4 + 31) / 32, rpb = 8 / wpr;
+  const int rblocks = (n2 + rpb - 1) / rpb, smem = CPB * (n2 + 1) * (int)sizeof(double);
+  auto k = digit_fold_kernel<Tin, CPB>;
+  if (smem > 48 * 1024) cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+  launch_pdl(k, dim3(rblocks + (n1 + CPB - 1) / CPB), dim3(256), smem, s, z, n1, n2, rblocks,
+             (const double*)p->near, pre, p->R.d, p->R.plane(), p->R.hk, p->exps, p->C.d, p->C.plane(), p->C.hk,
+             p->exps + n2, p->err, gate);
+}
+
+template <typename Tin>
+void digit_apply_M(DigitOperator* p, const Tin* z, double* w, const uint8_t* phi, double pen, double* pre,
+                   const int* gate, cudaStream_t s) {
+  const int n1 = p->n1, n2 = p->n2;
+  if (n1 >= 4 * kNumSMs) launch_fold<Tin, 4>(p, z, pre, gate, s);
+  else launch_fold<Tin, 2>(p, z, pre, gate, s);
+  DigitEpiParams ep{};
+  ep.rexp = p->exps;
+  ep.kexp_dev = p->kexp;
+  ep.row_b = 1 << 30;
+  ep.pre = pre;
+  ep.out0 = pre;
+  ep.ldo = n1;
+  launch_digit<DG_ROWS>(p, p->Tx, p->R, n1, 0, ep, gate, s);
+  ep.rexp = p->exps + n2;
+  ep.kexp_dev = p->kexp + 1;
+  ep.out0 = w;
+  ep.phi = phi;
+  ep.z = z;
+  ep.z_float = sizeof(Tin) == 4;
+  ep.pen = pen;
+  launch_digit<DG_COLS>(p, p->C, p->Ty, n2, 0, ep, gate, s);
+}
+template void digit_apply_M<double>(DigitOperator*, const double*, double*, const uint8_t*, double, double*,
+                                    const int*, cudaStream_t);
+template void digit_apply_M<float>(DigitOperator*, const float*, double*, const uint8_t*, double, double*, const int*,
+                                   cudaStream_t);
 
 template void digit_precond<double>(DigitPlan*, const double*, const double*, double*, const uint8_t*, double*,
                                     double*, double*, const int*, cudaStream_t);

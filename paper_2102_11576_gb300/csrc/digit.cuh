@@ -60,7 +60,9 @@ enum DigitEpi {
   DG_FIXED = 0,     // W of out^T, and the largest exponent of every row of out^T
   DG_QUOTIENT = 1,  // the same, with bounds of the exponents of both quotients of Eq. 4.6's tau divides
   DG_STORE = 2,     // out^T in FP64
-  DG_COMBINE = 3    // masked combine of Eq. 4.6 into z (FP64)
+  DG_COMBINE = 3,   // masked combine of Eq. 4.6 into z (FP64)
+  DG_ROWS = 4,      // the operands' roles swapped (A the matrix's pairs, S the rows of z): out = pre - product
+  DG_COLS = 5       // out = pre - product^T + (dt/eta) phi z, in FP64
 };
 
 struct DigitEpiParams {
@@ -77,6 +79,11 @@ struct DigitEpiParams {
   const double* inv0;  // DG_QUOTIENT: 1 / (1 - lx - ly) and 1 / (1 + dt/eta - lx - ly) at [n * M + m]
   const double* inv1;
   const uint8_t* phi;  // DG_COMBINE: out0[n * ldo + x] from channel phi[n * ldo + x]
+  const int* kexp_dev; // if set, added to kexp
+  const double* pre;   // DG_ROWS, DG_COLS
+  const void* z;       // DG_COLS: z (FP32 if z_float)
+  int z_float;
+  double pen;          // dt/eta
   long long wait_cycles;
 };
 
@@ -256,6 +263,10 @@ __global__ void __launch_bounds__(kDgThreads, 1)
   const bool mvalid = m < ep.M;
   const uint32_t tb = taddr + ((uint32_t)(q4 * 32) << 16) + (uint32_t)c0;
   const bool live = n0 + c0 < ep.N;  // this warp's columns reach into the matrix
+  // the row's exponent (DG_ROWS: lane l has column c0 + l's), read ahead of the main loop
+  const int E = EPI == DG_ROWS ? (lane < CW && n0 + c0 + lane < ep.N ? __ldg(ep.rexp + n0 + c0 + lane) : kDgNone)
+                               : (mvalid ? __ldg(ep.rexp + m) : kDgNone);
+  const int kdev = ep.kexp_dev ? __ldg(ep.kexp_dev) : 0;
   bool ok = true;
   long long u[kBoth ? 2 : CW];
   DgRaw raw;
@@ -357,8 +368,7 @@ __global__ void __launch_bounds__(kDgThreads, 1)
   // err[0]: a wait of this application's launches gave up; err[1]: one did since the host last looked
   const bool bad = !ok || *(volatile int*)err != 0;
   if (bad && lane == 0) atomicExch(err + 1, 1);
-  const int E = mvalid ? __ldg(ep.rexp + m) : kDgNone;
-  const int kx = E + ep.kexp;
+  const int kexp = ep.kexp + kdev, kx = E + kexp;
   const bool nan = bad || E == kDgNan;  // an incomplete tile, or a row that held an infinity or NaN
   const bool ch = m >= ep.row_b;
   const int mm = ch ? m - ep.row_b : m;
@@ -374,6 +384,26 @@ __global__ void __launch_bounds__(kDgThreads, 1)
   }
 #pragma unroll 1
   for (int c = 0; c < CW && n0 + c0 + c < ep.N; c += 2) {
+    // what the outputs read, in flight during the sums
+    constexpr bool kPre = EPI == DG_ROWS || EPI == DG_COLS, kPhi = EPI == DG_COLS || EPI == DG_COMBINE;
+    double pre[2][2];
+    uint8_t phi[2][2];
+    uint32_t inv[2][2][2];
+#pragma unroll
+    for (int q = 0; q < 2; ++q)
+#pragma unroll
+      for (int mir = 0; mir < 2; ++mir) {
+        const int n = n0 + c0 + c + q;
+        if (!mvalid || n >= ep.N) continue;
+        const size_t o = EPI == DG_ROWS ? (size_t)n * ep.ldo + (mir ? ep.n_full - 1 - m : m)
+                                        : (size_t)(mir ? ep.n_full - 1 - n : n) * ep.ldo + mm;
+        if constexpr (kPre) pre[q][mir] = ep.pre[o];
+        if constexpr (kPhi) phi[q][mir] = ep.phi[o];
+        if constexpr (EPI == DG_QUOTIENT) {  // (ldo = M)
+          inv[q][mir][0] = __ldg(reinterpret_cast<const uint32_t*>(ep.inv0 + o) + 1);
+          inv[q][mir][1] = __ldg(reinterpret_cast<const uint32_t*>(ep.inv1 + o) + 1);
+        }
+      }
     DgRaw next;
     if constexpr (kBoth) {
       dg_load2<BN>(tb + (uint32_t)c, raw);
@@ -394,17 +424,25 @@ __global__ void __launch_bounds__(kDgThreads, 1)
       for (int mir = 0; mir < 2; ++mir) {
         const int nn = mir ? ep.n_full - 1 - n : n;
         const long long w = mir ? u[q] - e : u[q] + e;
+        if constexpr (EPI == DG_ROWS) {  // pairs along m, the scale along n
+          const int En = __shfl_sync(0xffffffffu, E, c + q);
+          if (mvalid) {
+            const size_t o = (size_t)n * ep.ldo + (mir ? ep.n_full - 1 - m : m);
+            // (the middle pairs with itself: written once)
+            if (!(mir && 2 * m + 1 == ep.n_full))
+              static_cast<double*>(ep.out0)[o] = (bad || En == kDgNan) ? __longlong_as_double(0x7FF8000000000000ll)
+                                                                      : pre[q][mir] - dg_value(w, En + kexp);
+          }
+          continue;
+        }
         if constexpr (EPI == DG_FIXED || EPI == DG_QUOTIENT) {
           long long* __restrict__ out = static_cast<long long*>(ch ? ep.out1 : ep.out0);
           if (mvalid) out[(size_t)nn * ep.ldo + mm] = w;
           int x = nan ? kDgNan : dg_fixed_exponent(w, kx), x0 = kDgNone, x1 = kDgNone;
           if constexpr (EPI == DG_QUOTIENT) {
             if (mvalid) {  // |W inv| < 2^(x - 1022) 2^(e - 1022), e the biased exponent of inv
-              const size_t o = (size_t)nn * ep.M + m;
-              x0 = nan ? kDgNan
-                       : x + (int)((__ldg(reinterpret_cast<const uint32_t*>(ep.inv0 + o) + 1) >> 20) & 0x7FF) - 1022;
-              x1 = nan ? kDgNan
-                       : x + (int)((__ldg(reinterpret_cast<const uint32_t*>(ep.inv1 + o) + 1) >> 20) & 0x7FF) - 1022;
+              x0 = nan ? kDgNan : x + (int)((inv[q][mir][0] >> 20) & 0x7FF) - 1022;
+              x1 = nan ? kDgNan : x + (int)((inv[q][mir][1] >> 20) & 0x7FF) - 1022;
             }
             x0 = __reduce_max_sync(0xffffffffu, x0);
             x1 = __reduce_max_sync(0xffffffffu, x1);
@@ -420,7 +458,17 @@ __global__ void __launch_bounds__(kDgThreads, 1)
         } else {
           double* __restrict__ out = static_cast<double*>(ep.out0);
           const size_t o = (size_t)nn * ep.ldo + mm;
-          if (mvalid && (EPI == DG_STORE || (ep.phi[o] != 0) == ch))
+          if constexpr (EPI == DG_COLS) {
+            if (mvalid) {
+              double v = pre[q][mir] - dg_value(w, kx);
+              if (phi[q][mir])
+                v = __fma_rn(ep.pen,
+                             ep.z_float ? f64_exact(static_cast<const float*>(ep.z)[o])
+                                        : static_cast<const double*>(ep.z)[o],
+                             v);
+              out[o] = nan ? __longlong_as_double(0x7FF8000000000000ll) : v;
+            }
+          } else if (mvalid && (EPI == DG_STORE || (phi[q][mir] != 0) == ch))
             out[o] = nan ? __longlong_as_double(0x7FF8000000000000ll) : dg_value(w, kx);
         }
       }

@@ -211,6 +211,20 @@ void digit_precond(DigitPlan* p, const Tin* v, const double* vscale, double* z, 
 // out = (S_{n2} (x) S_{n1}) v in four launches; t: N doubles of scratch
 void digit_dst2(DigitPlan* p, const double* v, double* out, double* t, cudaStream_t s);
 
+// The FP64 operator w = M z as digit products (three launches): pre N doubles of
+// scratch.  Tables from the Toeplitz columns (digit_operator_params:
+// false if no scale keeps the sums exact).
+struct DigitOperator;
+int digit_operator_create(DigitOperator** out, int n1, int n2, cudaStream_t s);
+void digit_operator_destroy(DigitOperator* p);
+bool digit_operator_params(DigitOperator* p, const std::vector<double>& tx, const std::vector<double>& ty,
+                           cudaStream_t s);
+int digit_operator_error(DigitOperator* p, cudaStream_t s);
+void digit_operator_set_wait(DigitOperator* p, long long cycles);
+template <typename Tin>
+void digit_apply_M(DigitOperator* p, const Tin* z, double* w, const uint8_t* phi, double pen, double* pre,
+                   const int* gate, cudaStream_t s);
+
 // ---- batched instances: one launch per phase over every instance -------------
 // One instance of a batch as the multi-instance kernels see it (an array of
 // these lives in device memory).  Every buffer is the instance's own

@@ -1,4 +1,4 @@
-"""The FP64 sine transforms and preconditioner as digit products on the tensor
+"""The FP64 sine transforms, preconditioner and operator as digit products on the tensor
 cores, at the edges of their tiles (16, 32, 64 columns, 128 rows, 64-wide K
 slices) and up to the largest side they take, against dense extended-precision
 products.
@@ -9,7 +9,9 @@ one unit of W; W has at least 50 bits where the operand's row has its largest
 entry (n = 1), so 2^-51 at most; the sine matrix is within 2^-55.  Two products: below
 4 * 2^-51 = 1.8e-15.  The preconditioner: four products, 8 * 2^-51, the
 reciprocal and its product, 2 * 2^-53, and the rounded denominators, 2 * 2^-53:
-4.0e-15."""
+4.0e-15.  The operator: the middle diagonals in FP64 (six roundings of at most
+2^-53 of the coefficients' sum times the largest norm they meet) and two products
+of the rest, whose coefficients are at most 1/48 of that sum: 8 * 2^-53."""
 import numpy as np
 import pytest
 
@@ -59,6 +61,40 @@ def test_products_at_tile_edges(n1, n2):
         if sel.any():  # each channel against its own scale (the penalised one is far smaller)
             assert np.abs(z - ref)[sel].max() <= 4.0e-15 * np.sqrt((ref ** 2).sum())
     s.close()
+
+
+@pytest.mark.parametrize("n1,n2", SIZES)
+def test_operator_at_tile_edges(n1, n2):
+    w = workloads.random_problem(43, n1, n2)
+    s = solver(w)
+    v = torch.as_tensor(w["field"]).cuda()
+    t, pen, z = s.tables(), np.longdouble(s.params()["pen"]), w["field"].astype(np.longdouble)
+    Tx, Ty = (t[k].astype(np.longdouble)[np.abs(np.subtract.outer(np.arange(n), np.arange(n)))]
+              for k, n in (("t_x", n1), ("t_y", n2)))
+    out = w["in_omega"] == 0
+    ref = z - z @ Tx - Ty @ z + pen * out * z
+    err = s.apply_M(v).cpu().numpy() - ref
+    scale = 1 + 2 * (np.abs(t["t_x"]).sum() + np.abs(t["t_y"]).sum())
+    norm = np.sqrt((z ** 2).sum())
+    assert np.sqrt((err[~out] ** 2).sum()) <= 8 * 2.0 ** -53 * scale * norm
+    assert np.sqrt((err[out] ** 2).sum()) <= 8 * 2.0 ** -53 * (scale + float(pen)) * norm
+    assert torch.equal(s.apply_M(v * 2.0 ** 40), s.apply_M(v) * 2.0 ** 40)
+    v[n2 // 2, n1 // 2] = float("nan")
+    assert s.apply_M(v).isnan()[n2 // 2].all()
+    s.close()
+
+
+def test_operator_follows_new_parameters_in_a_captured_solve():
+    w = workloads.random_problem(44, 75, 52)
+    s = solver(w)
+    b = torch.as_tensor(w["field"]).cuda()
+    s.solve(b)
+    s.set_params(40.0 * w["kx"], 0.02 * w["ky"], w["dt"])
+    fresh = solver(dict(w, kx=40.0 * w["kx"], ky=0.02 * w["ky"]))
+    assert torch.equal(s.apply_M(b), fresh.apply_M(b))
+    assert torch.equal(s.solve(b)[0], fresh.solve(b)[0])
+    s.close()
+    fresh.close()
 
 
 def test_scaling_zeros_and_non_finite_entries():
