@@ -96,7 +96,7 @@ __device__ __forceinline__ void split_store(__nv_bfloat16* hi, __nv_bfloat16* lo
 // BF16 (one CTA per SM) runs sixteen warps, four per quarter; plain BF16 (two
 // CTAs per SM) eight.  With two tiles per CTA (TPC = 2, split BF16 only) the
 // second tile's K slices stream into a second pair of TMEM accumulators while
-// warps 2..15 run the first tile's epilogue, so the tensor pipe does not wait
+// warps 3..15 run the first tile's epilogue, so the tensor pipe does not wait
 // for it; all sixteen run the last one.
 __host__ __device__ constexpr int gemm_threads(int NT) { return NT == 3 ? 512 : 256; }
 //

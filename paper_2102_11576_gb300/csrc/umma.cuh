@@ -137,24 +137,8 @@ __device__ __forceinline__ uint64_t umma_desc_sw128(uint32_t smem_addr) {
   return d;
 }
 
-// 32 lanes x 32 consecutive 32-bit columns of tensor memory into registers
-// (warp w of the block reads lanes 32w .. 32w+31).
-__device__ __forceinline__ void tmem_ld32(uint32_t taddr, float* v) {
-  uint32_t r[32];
-  asm volatile(
-      "tcgen05.ld.sync.aligned.32x32b.x32.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, "
-      "%15, %16, %17, %18, %19, %20, %21, %22, %23, %24, %25, %26, %27, %28, %29, %30, %31}, [%32];"
-      : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
-        "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15]),
-        "=r"(r[16]), "=r"(r[17]), "=r"(r[18]), "=r"(r[19]), "=r"(r[20]), "=r"(r[21]), "=r"(r[22]), "=r"(r[23]),
-        "=r"(r[24]), "=r"(r[25]), "=r"(r[26]), "=r"(r[27]), "=r"(r[28]), "=r"(r[29]), "=r"(r[30]), "=r"(r[31])
-      : "r"(taddr));
-  asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-#pragma unroll
-  for (int i = 0; i < 32; ++i) v[i] = __uint_as_float(r[i]);
-}
-
-// Two such loads (columns c0 and c1) in flight before one wait.
+// 32 lanes x 32 consecutive 32-bit columns of tensor memory at c0 and at c1 into
+// registers (warp w of the block reads lanes 32 (w mod 4) ..), one wait.
 __device__ __forceinline__ void tmem_ld32x2(uint32_t c0, uint32_t c1, float* v0, float* v1) {
   uint32_t r[32], t[32];
 #define RSFDE_TMEM_LD(dst, addr)                                                                                  \
@@ -175,6 +159,29 @@ __device__ __forceinline__ void tmem_ld32x2(uint32_t c0, uint32_t c1, float* v0,
   for (int i = 0; i < 32; ++i) {
     v0[i] = __uint_as_float(r[i]);
     v1[i] = __uint_as_float(t[i]);
+  }
+}
+
+// 32 lanes x 16 columns at c0, and (TWO) 16 at c1, one wait.
+template <bool TWO>
+__device__ __forceinline__ void tmem_ld16(uint32_t c0, uint32_t c1, float* v0, float* v1) {
+  uint32_t r[16], t[16];
+#define RSFDE_TMEM_LD16(dst, addr)                                                                              \
+  asm volatile(                                                                                                 \
+      "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, " \
+      "%15}, [%16];"                                                                                            \
+      : "=r"(dst[0]), "=r"(dst[1]), "=r"(dst[2]), "=r"(dst[3]), "=r"(dst[4]), "=r"(dst[5]), "=r"(dst[6]),       \
+        "=r"(dst[7]), "=r"(dst[8]), "=r"(dst[9]), "=r"(dst[10]), "=r"(dst[11]), "=r"(dst[12]), "=r"(dst[13]),   \
+        "=r"(dst[14]), "=r"(dst[15])                                                                            \
+      : "r"(addr))
+  RSFDE_TMEM_LD16(r, c0);
+  if (TWO) RSFDE_TMEM_LD16(t, c1);
+#undef RSFDE_TMEM_LD16
+  asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+#pragma unroll
+  for (int i = 0; i < 16; ++i) {
+    v0[i] = __uint_as_float(r[i]);
+    if (TWO) v1[i] = __uint_as_float(t[i]);
   }
 }
 
