@@ -671,7 +671,7 @@ void enqueue_rhs(rsfde_ctx* c, const double* u, const double* uu, const double* 
 // Krylov basis element type Tv: double, df or float (basis_kind).
 template <typename Tz, typename Tv>
 void enqueue_cycle_t(rsfde_ctx* c) {
-  const size_t N = c->N;
+  const size_t N = c->N, ld = basis_ld(N);
   const int m = c->opts.restart;
   const int* gi = &c->st->run_iter;
   const int* gc = &c->st->run_cycle;
@@ -682,12 +682,11 @@ void enqueue_cycle_t(rsfde_ctx* c) {
   // pair hi, lo) as the first GEMM operand of iteration j+1, whose split pass
   // is then skipped.
   Bf16Out bo{};
-  constexpr int kVec = 16 / sizeof(Tv);
+  constexpr int kVec = std::is_same<Tv, float>::value ? 4 : 1;
   const bool fused = (std::is_same<Tv, float>::value || std::is_same<Tv, double>::value) &&
-                     c->opts.use_precond && bf16_precond_on(c) && N % kVec == 0 &&
-                     bf16_plan_a0(c->bf16, kVec, &bo);
+                     c->opts.use_precond && bf16_precond_on(c) && bf16_plan_a0(c->bf16, kVec, &bo);
   for (int j = 0; j < m; ++j) {
-    const Tv* vj = V + (size_t)j * N;
+    const Tv* vj = V + (size_t)j * ld;
     Tz* zj = Z + (size_t)j * N;
     if (c->opts.use_precond) {
       if (bf16_precond_on(c))
@@ -702,7 +701,7 @@ void enqueue_cycle_t(rsfde_ctx* c) {
       ProfScope ps(c, RSFDE_K_OTHER);
       launch_scale_copy<Tv, Tz>(vj, &c->st->s[j], zj, N, gi, c->stream);  // P = I: z_j = v_j
     }
-    Tv* w = V + (size_t)(j + 1) * N;
+    Tv* w = V + (size_t)(j + 1) * ld;
     if constexpr (std::is_same<Tv, df>::value) enqueue_apply_M_t<df, Tz, df>(c, zj, w, gi, c->xdf.tab, c->ydf.tab);
     else if constexpr (std::is_same<Tv, float>::value)
       enqueue_apply_M_t<float, Tz, float>(c, zj, w, gi, c->x32.tab, c->y32.tab);
@@ -732,13 +731,13 @@ void enqueue_cycle_t(rsfde_ctx* c) {
 // One cycle of left-preconditioned GMRES(m) (Section 5): w = P^-1 M v_j,
 // the same Gram-Schmidt and Givens kernels, x += V y, residual P^-1 (b - M x).
 void enqueue_cycle_left(rsfde_ctx* c) {
-  const size_t N = c->N;
+  const size_t N = c->N, ld = basis_ld(N);
   const int m = c->opts.restart;
   const int* gi = &c->st->run_iter;
   double* tmp = static_cast<double*>(c->Z);  // Z is unused by this variant
   for (int j = 0; j < m; ++j) {
-    const double* vj = c->V + (size_t)j * N;
-    double* w = c->V + (size_t)(j + 1) * N;
+    const double* vj = c->V + (size_t)j * ld;
+    double* w = c->V + (size_t)(j + 1) * ld;
     if (c->opts.use_precond) {
       enqueue_apply_M<double>(c, vj, tmp, gi);    // M V_j
       enqueue_precond64(c, tmp, &c->st->s[j], w, gi);  // P^-1 M v_j
@@ -753,10 +752,10 @@ void enqueue_cycle_left(rsfde_ctx* c) {
     for (int pass = 0; pass < (cgs2 ? 2 : 1); ++pass) {
       {
         ProfScope ps(c, RSFDE_K_MULTIDOT);
-        launch_multidot<double>(c->V, N, j, pass, c->partials, c->st, c->stream);
+        launch_multidot_paper(c->V, N, j, pass, c->partials, c->st, c->stream);
       }
       ProfScope ps(c, RSFDE_K_UPDATE);
-      launch_update<double>(c->V, N, j, (!cgs2 || pass == 1) ? 1 : 0, c->partials, c->st, c->stream);
+      launch_update_paper(c->V, N, j, (!cgs2 || pass == 1) ? 1 : 0, c->partials, c->st, c->stream);
     }
   }
   {
@@ -1339,7 +1338,7 @@ int setup_multi(rsfde_batch* b) {
       // as the single-instance cycle: the basis update writes the next
       // operand when the plan takes it (enqueue_cycle_t's `fused`)
       Bf16Out bo{};
-      I.a0_fused = (c->N % 2 == 0 && bf16_plan_a0(c->bf16, 2, &bo)) ? 1 : 0;
+      I.a0_fused = bf16_plan_a0(c->bf16, 1, &bo) ? 1 : 0;
       bf16_plan_a0_any(c->bf16, &bo);
       I.a0 = bo.a0;
       I.a0_lo = bo.lo;
@@ -1701,14 +1700,16 @@ int rsfde_setup(rsfde_ctx** out, const rsfde_grid* g, const uint8_t* mask, doubl
   c->dt = dt;
   c->eta = eta;
   const size_t N = c->N, m = o.restart;
-  c->npartials = (size_t)(kMaxRestart + 2) * (size_t)vec_grid(N);
+  // (a reduction has at most one block per kBlock elements, and eight per SM)
+  const size_t per_vec = (N + kBlock - 1) / kBlock, grid_cap = (size_t)kNumSMs * 8;
+  c->npartials = (size_t)(kMaxRestart + 2) * (per_vec < grid_cap ? per_vec : grid_cap);
   if (c->npartials < (size_t)kMaxPartials) c->npartials = kMaxPartials;
   cudaError_t e = cudaSuccess;
   auto alloc = [&](void** p, size_t bytes) {
     if (e == cudaSuccess) e = cudaMalloc(p, bytes);
   };
   alloc((void**)&c->phi, N);
-  alloc((void**)&c->V, (m + 1) * N * sizeof(double));
+  alloc((void**)&c->V, (m + 1) * basis_ld(N) * sizeof(double));
   alloc(&c->Z, m * N * sizeof(double));
   alloc((void**)&c->tmpx, N * sizeof(double));
   alloc(&c->T1, N * sizeof(double));

@@ -6,6 +6,10 @@
 namespace rsfde {
 
 constexpr int kMaxRestart = 64;  // largest m of FGMRES(m)
+// Distance of the Krylov basis' vectors (elements of any type): 16-byte packs
+// need every vector aligned, also of odd grids.  (One element at a time, the
+// FP64 update of 1201 x 777 ran at 61 % of the rate of 16-byte packs.)
+__host__ __device__ constexpr size_t basis_ld(size_t N) { return (N + 3) & ~(size_t)3; }
 
 // Programmatic dependent launch (the BF16 preconditioner's split and GEMM
 // chain).  A kernel launched by launch_pdl may be scheduled while the previous
@@ -128,6 +132,19 @@ __device__ __forceinline__ bool arrive_last(unsigned int* counter, unsigned int 
   __syncthreads();
   if (is_last) __threadfence();
   return is_last != 0;
+}
+
+// w 2^k as FP64, rounded to nearest, by integer instructions.
+__device__ __forceinline__ double ldexp_i64(long long w, int k) {
+  if (w == 0) return 0.0;
+  const unsigned long long s = (unsigned long long)w & (1ull << 63);
+  unsigned long long m = w < 0 ? 0ull - (unsigned long long)w : (unsigned long long)w;
+  const int z = __clzll((long long)m);
+  m <<= z;
+  const int e = 1023 + 63 - z + k;                              // biased exponent
+  const unsigned long long r = (m >> 11) + ((m >> 10) & 1ull);  // 2^52 <= r <= 2^53: a carry moves the exponent
+  if (e > 0 && e < 2046) return __longlong_as_double((long long)(s | (((unsigned long long)(e - 1) << 52) + r)));
+  return scalbn(__longlong_as_double((long long)(s | ((1022ull << 52) + r))), e - 1023);
 }
 
 // Sum of the `count` values p[0..count) by one warp in an order fixed by count

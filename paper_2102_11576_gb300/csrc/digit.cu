@@ -176,7 +176,7 @@ __global__ void __launch_bounds__(kBlock)
     const int p = 8 * c + k;
     q0[k] = q1[k] = 0;
     if (p < len && live) {
-      const double v = dg_value(src[o + p], __ldg(cexp + p) + kexp);
+      const double v = ldexp_i64(src[o + p], __ldg(cexp + p) + kexp);
       q0[k] = dg_quantize(v * __ldg(inv0 + o + p), E0);
       q1[k] = dg_quantize(v * __ldg(inv1 + o + p), E1);
     }

@@ -154,18 +154,6 @@ __device__ __forceinline__ long long dg_sum(const DgRaw& t, int q) {
   for (int s = 0; s < kDgDigits; ++s) g[s] = __float2int_rn(__uint_as_float(t.r[s][q]));
   return dg_sum(g);
 }
-// W 2^k as FP64, rounded to nearest, by integer instructions.
-__device__ __forceinline__ double dg_value(long long w, int k) {
-  if (w == 0) return 0.0;
-  const unsigned long long s = (unsigned long long)w & (1ull << 63);
-  unsigned long long m = w < 0 ? 0ull - (unsigned long long)w : (unsigned long long)w;
-  const int z = __clzll((long long)m);
-  m <<= z;
-  const int e = 1023 + 63 - z + k;                              // biased exponent
-  const unsigned long long r = (m >> 11) + ((m >> 10) & 1ull);  // 2^52 <= r <= 2^53: a carry moves the exponent
-  if (e > 0 && e < 2046) return __longlong_as_double((long long)(s | (((unsigned long long)(e - 1) << 52) + r)));
-  return scalbn(__longlong_as_double((long long)(s | ((1022ull << 52) + r))), e - 1023);
-}
 // E with |W 2^k| <= 2^(E - 1022), at least that of a W of 32 bits (which the
 // next split takes without loss).
 __device__ __forceinline__ int dg_fixed_exponent(long long w, int k) {
@@ -431,7 +419,7 @@ __global__ void __launch_bounds__(kDgThreads, 1)
             // (the middle pairs with itself: written once)
             if (!(mir && 2 * m + 1 == ep.n_full))
               static_cast<double*>(ep.out0)[o] = (bad || En == kDgNan) ? __longlong_as_double(0x7FF8000000000000ll)
-                                                                      : pre[q][mir] - dg_value(w, En + kexp);
+                                                                      : pre[q][mir] - ldexp_i64(w, En + kexp);
           }
           continue;
         }
@@ -460,7 +448,7 @@ __global__ void __launch_bounds__(kDgThreads, 1)
           const size_t o = (size_t)nn * ep.ldo + mm;
           if constexpr (EPI == DG_COLS) {
             if (mvalid) {
-              double v = pre[q][mir] - dg_value(w, kx);
+              double v = pre[q][mir] - ldexp_i64(w, kx);
               if (phi[q][mir])
                 v = __fma_rn(ep.pen,
                              ep.z_float ? f64_exact(static_cast<const float*>(ep.z)[o])
@@ -469,7 +457,7 @@ __global__ void __launch_bounds__(kDgThreads, 1)
               out[o] = nan ? __longlong_as_double(0x7FF8000000000000ll) : v;
             }
           } else if (mvalid && (EPI == DG_STORE || (phi[q][mir] != 0) == ch))
-            out[o] = nan ? __longlong_as_double(0x7FF8000000000000ll) : dg_value(w, kx);
+            out[o] = nan ? __longlong_as_double(0x7FF8000000000000ll) : ldexp_i64(w, kx);
         }
       }
     }

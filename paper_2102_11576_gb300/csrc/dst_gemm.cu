@@ -561,7 +561,7 @@ __global__ void __launch_bounds__(kBlock) split_multi_kernel(const BatchInst* __
     const BatchInst& I = bi[mi];
     if (j > 0 && I.a0_fused) continue;  // uniform over the block
     const int lb = vb - sact[mi], nb = __ldg(prefix + mi + 1) - __ldg(prefix + mi);
-    const double* v = I.V + (size_t)j * I.N;
+    const double* v = I.V + (size_t)j * basis_ld(I.N);
     const double sc = I.st->s[j];
     __nv_bfloat16* hi = static_cast<__nv_bfloat16*>(I.a0);
     __nv_bfloat16* lo = static_cast<__nv_bfloat16*>(I.a0_lo);

@@ -159,6 +159,7 @@ void launch_precond_rows(const T* T2a, const T* T2b, const uint8_t* phi, Tz* z, 
 // a0 + y*ld, even x at x/2, odd x at hk + x/2), the next preconditioner's first
 // operand; with lo set (split BF16) also the remainder bf16(x - hi) at the
 // same place of lo.
+// (the FP64 update takes any n1; the FP32 one n1 a multiple of its four elements a pack)
 struct Bf16Out {
   __nv_bfloat16* a0;
   __nv_bfloat16* lo;
@@ -441,6 +442,11 @@ void launch_multidot(const Tv* V, size_t N, int j, int accumulate, double* parti
 template <typename Tv>
 void launch_update(Tv* V, size_t N, int j, int final_pass, double* partials, SolverState* st, cudaStream_t s,
                    const Bf16Out* bo = nullptr);
+// the same for paper mode, which keeps its order of the sums
+void launch_multidot_paper(const double* V, size_t N, int j, int accumulate, double* partials, SolverState* st,
+                           cudaStream_t s);
+void launch_update_paper(double* V, size_t N, int j, int final_pass, double* partials, SolverState* st,
+                         cudaStream_t s);
 void launch_solve_y(SolverState* st, cudaStream_t s);
 template <typename Tz>
 void launch_xupdate(double* x, const Tz* Z, size_t N, SolverState* st, cudaStream_t s);

@@ -156,8 +156,9 @@ struct VecOps<df> {
 constexpr int kWarps = kBlock / 32;
 
 // VEC consecutive elements moved as one 16-byte access (VEC = 16 / sizeof(Tv));
-// VEC = 1: one element.  The 16-byte form needs every basis vector 16-byte
-// aligned, i.e. N * sizeof(Tv) a multiple of 16.
+// VEC = 1: one element.  The basis vectors are basis_ld(N) elements apart, so
+// each is 16-byte aligned; what N leaves over of the last pack is taken element by
+// element (tail_packs).
 template <typename Tv, int VEC>
 __device__ __forceinline__ void ld_vec(const Tv* p, Tv* o) {
   if constexpr (VEC == 1) {
@@ -191,16 +192,72 @@ __device__ __forceinline__ void st_vec(Tv* p, const Tv* v) {
   }
 }
 
-// Block sums of cnt <= K accumulators: warp sums, then warp k adds the
-// per-warp FP64 sums of accumulator k (fixed order).  Thread 32k returns sum k.
-//
-// FP64 with all K (2, 4 or 8) accumulators in use: the K warp sums by
-// recursive halving -- at the step over lane bit b a lane keeps half of its
-// partial sums and adds the partner's matching half, so after log2 K steps
-// each lane holds one accumulator's partial and the last 5 - log2 K steps
-// finish it: K - 1 + 5 - log2 K additions and shuffles per lane instead of
-// 5 K.  The pairs and their order are those of warp_sum (lane bits 4 down to
-// 0), so every sum is the same number.
+// The warp sums of K (1, 2, 4 or 8) FP64 accumulators per lane, on the integer
+// pipe: an FP64 addition holds a scheduler's FP64 pipe for 64 clocks, and a
+// block that sums few elements per thread spends as long on its warp sums as
+// on its products.  Accumulator i becomes integers q = round(x 2^(1080 - E)), E its
+// largest biased exponent over the warp: |q| < 2^58, so 32 of them add up
+// exactly; what is lost is half a unit of q per lane, 2^-59 of the largest
+// (FP64 additions: 2^-53 of every partial sum).  The additions by recursive
+// halving: at the step over lane bit b a lane keeps half of its sums and adds
+// the partner's matching half, so after log2 K steps each lane holds one
+// accumulator's partial and the last 5 - log2 K steps finish it.
+// A warp that holds an infinity or NaN takes FP64 additions.
+__device__ __forceinline__ long long fixed58(double x, int E) {  // E >= the biased exponent of x, E >= 1
+  const unsigned long long b = (unsigned long long)__double_as_longlong(x);
+  const int e = (int)(b >> 52) & 0x7FF;
+  const unsigned long long m = b & 0xFFFFFFFFFFFFFull;
+  const unsigned long long mag = e ? (m | (1ull << 52)) : m;
+  const int sh = E - (e ? e : 1) - 5;
+  const unsigned long long q = sh <= 0 ? mag << -sh : sh < 60 ? (mag + (1ull << (sh - 1))) >> sh : 0ull;
+  return (long long)b < 0 ? -(long long)q : (long long)q;
+}
+template <int K>
+__device__ __forceinline__ void warp_sums_f64(const double* acc, double (*sh)[kWarps], int w, int l) {
+  constexpr int R = K == 8 ? 3 : K == 4 ? 2 : K == 2 ? 1 : 0;
+  static_assert(K == 1 << R, "1, 2, 4 or 8 accumulators");
+  int e[K], top = 0;
+#pragma unroll
+  for (int i = 0; i < K; ++i) {
+    const int x = (__double2hiint(acc[i]) >> 20) & 0x7FF;
+    e[i] = (int)__reduce_max_sync(0xffffffffu, (unsigned)(x ? x : 1));
+    top = max(top, e[i]);
+  }
+  if (top == 2047) {
+#pragma unroll
+    for (int i = 0; i < K; ++i) {
+      const double ws = VecOps<double>::warp_sum(acc[i]);
+      if (l == 0) sh[i][w] = ws;
+    }
+    return;
+  }
+  long long v[K];
+#pragma unroll
+  for (int i = 0; i < K; ++i) v[i] = fixed58(acc[i], e[i]);
+#pragma unroll
+  for (int s = 0; s < R; ++s) {
+    const int off = 16 >> s;
+    constexpr int kMax = K >> 1;
+    const bool up = (l & off) != 0;  // keep the upper half of the current K >> s values
+#pragma unroll
+    for (int i = 0; i < kMax; ++i) {
+      const int half = (K >> s) >> 1;
+      if (i < half) {
+        const long long send = up ? v[i] : v[half + i];
+        const long long keep = up ? v[half + i] : v[i];
+        v[i] = keep + __shfl_xor_sync(0xffffffffu, send, off);
+        e[i] = up ? e[half + i] : e[i];
+      }
+    }
+  }
+#pragma unroll
+  for (int off = 16 >> R; off; off >>= 1) v[0] += __shfl_xor_sync(0xffffffffu, v[0], off);
+  if ((l & ((32 >> R) - 1)) == 0) sh[l >> (5 - R)][w] = ldexp_i64(v[0], e[0] - 1080);  // accumulator l >> (5 - R)
+}
+// The same K sums by FP64 additions (the pairs and their order those of warp_sum),
+// for paper mode: its stop test, ||P^-1 (b - M x)|| at 1e-8, is near what FP64 resolves of
+// the penalty rows, so another rounding of the sums moves its solutions by as much as
+// their error (128 x 128: 9.4e-8 against 2.0e-7), and its sums stay as they were.
 template <int K>
 __device__ __forceinline__ void warp_sums_halving(const double* acc, double (*sh)[kWarps], int w, int l) {
   constexpr int R = K == 8 ? 3 : K == 4 ? 2 : 1;
@@ -226,25 +283,26 @@ __device__ __forceinline__ void warp_sums_halving(const double* acc, double (*sh
   for (int off = 16 >> R; off; off >>= 1) v[0] += __shfl_xor_sync(0xffffffffu, v[0], off);
   if ((l & ((32 >> R) - 1)) == 0) sh[l >> (5 - R)][w] = v[0];  // accumulator l >> (5 - R)
 }
-template <typename Tv, int K>
+
+// Block sums of cnt <= K accumulators (the others zero): warp sums, then warp k
+// adds the per-warp FP64 sums of accumulator k (fixed order).  Thread 32k
+// returns sum k.  PAPER: paper mode's FP64 additions.
+template <typename Tv, int K, bool PAPER>
 __device__ __forceinline__ double block_sums(const Tv* acc, int cnt, double (*sh)[kWarps]) {
   const int w = threadIdx.x >> 5, l = threadIdx.x & 31;
-  if constexpr (std::is_same<Tv, double>::value && (K == 2 || K == 4 || K == 8)) {
-    if (cnt == K) {
-      warp_sums_halving<K>(acc, sh, w, l);
-    } else {
-#pragma unroll
-      for (int k = 0; k < K; ++k) {
-        if (k < cnt) {
-          const double ws = VecOps<Tv>::warp_sum(acc[k]);
-          if (l == 0) sh[k][w] = ws;
-        }
+  if constexpr (std::is_same<Tv, double>::value && !PAPER) {
+    warp_sums_f64<K>(acc, sh, w, l);
+  } else {
+    bool done = false;
+    if constexpr (PAPER && K > 1) {
+      if (cnt == K) {
+        warp_sums_halving<K>(acc, sh, w, l);
+        done = true;
       }
     }
-  } else {
 #pragma unroll
     for (int k = 0; k < K; ++k) {
-      if (k < cnt) {
+      if (!done && k < cnt) {
         const double ws = VecOps<Tv>::warp_sum(acc[k]);
         if (l == 0) sh[k][w] = ws;
       }
@@ -253,10 +311,19 @@ __device__ __forceinline__ double block_sums(const Tv* acc, int cnt, double (*sh
   __syncthreads();
   double v = 0.0;
   if (w < cnt) {
-    v = l < kWarps ? sh[w][l] : 0.0;
-    v = VecOps<double>::warp_sum(v);
+    v = sh[w][l & (kWarps - 1)];
+#pragma unroll
+    for (int o = kWarps / 2; o; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
   }
   return v;
+}
+
+// The N mod VEC elements after the last whole pack belong to the thread whose
+// next pack would be that one.
+template <int VEC>
+__device__ __forceinline__ bool owns_tail(size_t N, int bid, int nblk) {
+  if (VEC == 1 || N % VEC == 0) return false;
+  return bid * (size_t)blockDim.x + threadIdx.x == (N / VEC) % ((size_t)nblk * blockDim.x);
 }
 
 // Partial sums acc[k] += <w, V_{i0+k}> over this thread's packs for exactly
@@ -268,7 +335,7 @@ template <typename Tv, int VEC, int C, int UNR>
 __device__ __forceinline__ void dot_rounds(const Tv* __restrict__ V, const Tv* __restrict__ w, size_t N, int i0,
                                            Tv* acc, int bx, int nbx) {
   using Op = VecOps<Tv>;
-  const size_t NP = N / VEC;  // VEC divides N (launcher)
+  const size_t NP = N / VEC, ld = basis_ld(N);
   const size_t stride = (size_t)nbx * blockDim.x;
   for (size_t q0 = bx * (size_t)blockDim.x + threadIdx.x; q0 < NP; q0 += UNR * stride) {
     Tv wv[UNR][VEC];
@@ -286,7 +353,7 @@ __device__ __forceinline__ void dot_rounds(const Tv* __restrict__ V, const Tv* _
 #pragma unroll
       for (int k = 0; k < C; ++k) {
         if (in) {
-          ld_vec<Tv, VEC>(V + (size_t)(i0 + k) * N + q * VEC, a[u][k]);
+          ld_vec<Tv, VEC>(V + (size_t)(i0 + k) * ld + q * VEC, a[u][k]);
         } else {
 #pragma unroll
           for (int e = 0; e < VEC; ++e) a[u][k][e] = Op::zero();
@@ -308,7 +375,7 @@ __device__ __forceinline__ void dot_rounds(const Tv* __restrict__ V, const Tv* _
 // L2).  The chunk's exact count selects the unrolled body (dot_rounds).
 // accumulate = 1 adds to H (second CGS pass).  The last block finishes the
 // j+1 sums, one warp per sum.
-template <typename Tv, int VEC, int CH>
+template <typename Tv, int VEC, int CH, bool PAPER>
 __device__ __forceinline__ void multidot_body(const Tv* __restrict__ V, size_t N, int j, int accumulate,
                                               double* partials, SolverState* st, int bx, int nbx, int by, int nby) {
   if (closed(&st->run_iter)) return;
@@ -318,7 +385,7 @@ __device__ __forceinline__ void multidot_body(const Tv* __restrict__ V, size_t N
   const int per = (j + 1 + nby - 1) / nby;  // <= CH (launcher)
   const int i0 = by * per;
   const int cnt = min(per, j + 1 - i0);
-  const Tv* __restrict__ w = V + (size_t)(j + 1) * N;
+  const Tv* __restrict__ w = V + (size_t)(j + 1) * basis_ld(N);
   Tv acc[CH];
 #pragma unroll
   for (int k = 0; k < CH; ++k) acc[k] = Op::zero();
@@ -339,8 +406,16 @@ __device__ __forceinline__ void multidot_body(const Tv* __restrict__ V, size_t N
     default:
       break;
   }
+  if (owns_tail<VEC>(N, bx, nbx)) {
+    for (size_t p = N / VEC * VEC; p < N; ++p) {
+      const Tv wp = Op::ld(w + p);
+#pragma unroll
+      for (int k = 0; k < CH; ++k)
+        if (k < cnt) acc[k] = Op::fma(acc[k], wp, Op::ld(V + (size_t)(i0 + k) * basis_ld(N) + p));
+    }
+  }
   const int G = nbx;
-  const double bs = block_sums<Tv, CH>(acc, cnt, wsum);
+  const double bs = block_sums<Tv, CH, PAPER>(acc, cnt, wsum);
   const int wk = threadIdx.x >> 5;
   if ((threadIdx.x & 31) == 0 && wk < cnt) partials[(size_t)(i0 + wk) * G + bx] = bs;
   if (arrive_last(&st->counter, nbx * nby)) {
@@ -355,17 +430,17 @@ __device__ __forceinline__ void multidot_body(const Tv* __restrict__ V, size_t N
     }
   }
 }
-template <typename Tv, int VEC, int CH>
+template <typename Tv, int VEC, int CH, bool PAPER>
 __global__ void __launch_bounds__(kBlock) multidot_kernel(const Tv* __restrict__ V, size_t N, int j, int accumulate,
                                                           double* partials, SolverState* st) {
-  multidot_body<Tv, VEC, CH>(V, N, j, accumulate, partials, st, blockIdx.x, gridDim.x, blockIdx.y, gridDim.y);
+  multidot_body<Tv, VEC, CH, PAPER>(V, N, j, accumulate, partials, st, blockIdx.x, gridDim.x, blockIdx.y, gridDim.y);
 }
 
 // Loads chunk k < C of the basis (vectors i0 .. i0+C-1) for UNR packs, then
 // subtracts them from val in the order i0, i0+1, ...; every load is issued
 // before the dependent chains.
 template <typename Tv, int VEC, int C, int UNR>
-__device__ __forceinline__ void update_chunk(const Tv* __restrict__ V, size_t N, size_t NP, size_t q0,
+__device__ __forceinline__ void update_chunk(const Tv* __restrict__ V, size_t ld, size_t NP, size_t q0,
                                              size_t stride, int i0, const Tv* ncoef, Tv (&val)[UNR][VEC]) {
   using Op = VecOps<Tv>;
   Tv a[UNR][C][VEC];
@@ -375,7 +450,7 @@ __device__ __forceinline__ void update_chunk(const Tv* __restrict__ V, size_t N,
 #pragma unroll
     for (int k = 0; k < C; ++k) {
       if (in) {
-        ld_vec<Tv, VEC>(V + (size_t)(i0 + k) * N + (q0 + u * stride) * VEC, a[u][k]);
+        ld_vec<Tv, VEC>(V + (size_t)(i0 + k) * ld + (q0 + u * stride) * VEC, a[u][k]);
       } else {
 #pragma unroll
         for (int e = 0; e < VEC; ++e) a[u][k][e] = Op::zero();
@@ -390,6 +465,28 @@ __device__ __forceinline__ void update_chunk(const Tv* __restrict__ V, size_t N,
       for (int e = 0; e < VEC; ++e) val[u][e] = Op::fma(val[u][e], ncoef[i0 + k], a[u][k][e]);
 }
 
+// Elements p .. p + VEC - 1 of an FP64 vector (rows of n1, any n1: a pack may end one row and
+// begin the next) as BF16, in the layout of the first GEMM's operand: even x to column
+// x/2, odd x to hk + x/2; lo: what is left of each.
+template <int VEC>
+__device__ __forceinline__ void write_a0(const Bf16Out& bo, size_t p, const double* v) {
+  int y = (int)((unsigned)p / (unsigned)bo.n1), x = (int)((unsigned)p - (unsigned)y * (unsigned)bo.n1);
+  size_t o = (size_t)y * bo.ld + (x >> 1);
+  if (VEC == 1 || (bo.n1 & 1)) o += (x & 1) ? bo.hk : 0;  // (a pack of even rows starts at an even x)
+#pragma unroll
+  for (int e = 0; e < VEC; ++e) {
+    const float f = f32_trunc(v[e]);
+    const __nv_bfloat16 h = __float2bfloat16_rn(f);
+    bo.a0[o] = h;
+    if (bo.lo) bo.lo[o] = __float2bfloat16_rn(f - __bfloat162float(h));
+    if (VEC == 1) break;
+    static_assert(VEC <= 2, "one or two FP64 elements");
+    if (!(bo.n1 & 1)) o += bo.hk;
+    else if (x + 1 == bo.n1) o = (size_t)(y + 1) * bo.ld;
+    else o = (x & 1) ? o - bo.hk + 1 : o + bo.hk;
+  }
+}
+
 // The update's sweep over this block's packs for j + 1 = nfull * CH + R basis
 // vectors: nfull chunks of CH, then a tail of R (a compile-time count, so no
 // multiply-add is issued for an empty slot -- the FP64 form is bound by the
@@ -400,9 +497,9 @@ __device__ __forceinline__ Tv update_rounds(Tv* __restrict__ V, size_t N, int j,
                                             const Tv* ncoef, const Bf16Out& bo, int bid, int nblk) {
   using Op = VecOps<Tv>;
   constexpr int UNR = kDotChunk / CH;
-  Tv* __restrict__ w = V + (size_t)(j + 1) * N;
+  const size_t NP = N / VEC, ld = basis_ld(N);
+  Tv* __restrict__ w = V + (size_t)(j + 1) * ld;
   Tv acc = Op::zero();
-  const size_t NP = N / VEC;  // VEC divides N (launcher)
   const size_t stride = (size_t)nblk * blockDim.x;
   for (size_t q0 = bid * (size_t)blockDim.x + threadIdx.x; q0 < NP; q0 += UNR * stride) {
     Tv val[UNR][VEC];
@@ -415,8 +512,8 @@ __device__ __forceinline__ Tv update_rounds(Tv* __restrict__ V, size_t N, int j,
         for (int e = 0; e < VEC; ++e) val[u][e] = Op::zero();
       }
     }
-    for (int c = 0; c < nfull; ++c) update_chunk<Tv, VEC, CH, UNR>(V, N, NP, q0, stride, c * CH, ncoef, val);
-    if constexpr (R > 0) update_chunk<Tv, VEC, R, UNR>(V, N, NP, q0, stride, nfull * CH, ncoef, val);
+    for (int c = 0; c < nfull; ++c) update_chunk<Tv, VEC, CH, UNR>(V, ld, NP, q0, stride, c * CH, ncoef, val);
+    if constexpr (R > 0) update_chunk<Tv, VEC, R, UNR>(V, ld, NP, q0, stride, nfull * CH, ncoef, val);
 #pragma unroll
     for (int u = 0; u < UNR; ++u) {
       const size_t q = q0 + u * stride;
@@ -439,19 +536,8 @@ __device__ __forceinline__ Tv update_rounds(Tv* __restrict__ V, size_t N, int j,
                 __floats2bfloat162_rn(val[u][1] - d.x, val[u][3] - d.y);
           }
         }
-      } else if constexpr (std::is_same<Tv, double>::value && VEC == 2) {
-        if (bo.a0 && final_pass) {  // x = p mod n1 is even (n1 is): x to column x/2, x+1 to hk + x/2
-          const int y = (int)(p / (size_t)bo.n1), x = (int)(p - (size_t)y * bo.n1);
-          const size_t o = (size_t)y * bo.ld + (x >> 1);
-          const float f0 = f32_trunc(val[u][0]), f1 = f32_trunc(val[u][1]);
-          const __nv_bfloat16 h0 = __float2bfloat16_rn(f0), h1 = __float2bfloat16_rn(f1);
-          bo.a0[o] = h0;
-          bo.a0[o + bo.hk] = h1;
-          if (bo.lo) {
-            bo.lo[o] = __float2bfloat16_rn(f0 - __bfloat162float(h0));
-            bo.lo[o + bo.hk] = __float2bfloat16_rn(f1 - __bfloat162float(h1));
-          }
-        }
+      } else if constexpr (std::is_same<Tv, double>::value) {
+        if (bo.a0 && final_pass) write_a0<VEC>(bo, p, val[u]);
       }
 #pragma unroll
       for (int e = 0; e < VEC; ++e) acc = Op::fma(acc, val[u][e], val[u][e]);
@@ -464,7 +550,7 @@ __device__ __forceinline__ Tv update_rounds(Tv* __restrict__ V, size_t N, int j,
 // the last block runs the Givens step.  The basis vectors are read in chunks
 // of CH independent loads for each of kDotChunk / CH packs ahead of the
 // dependent update chains (about eight loads in flight for every j).
-template <typename Tv, int VEC, int CH>
+template <typename Tv, int VEC, int CH, bool PAPER>
 __device__ __forceinline__ void update_body(Tv* __restrict__ V, size_t N, int j, int final_pass, double* partials,
                                             SolverState* st, const Bf16Out& bo, int bid, int nblk) {
   if (closed(&st->run_iter)) return;
@@ -492,17 +578,30 @@ __device__ __forceinline__ void update_body(Tv* __restrict__ V, size_t N, int j,
     default:
       break;
   }
-  const double bs = block_sums<Tv, 1>(&acc, 1, wsum);
+  if (owns_tail<VEC>(N, bid, nblk)) {
+    const size_t ld = basis_ld(N);
+    Tv* w = V + (size_t)(j + 1) * ld;
+    for (size_t p = N / VEC * VEC; p < N; ++p) {
+      Tv v = Op::ld(w + p);
+      for (int i = 0; i <= j; ++i) v = Op::fma(v, ncoef[i], Op::ld(V + (size_t)i * ld + p));
+      Op::st(w + p, v);
+      if constexpr (std::is_same<Tv, double>::value) {
+        if (bo.a0 && final_pass) write_a0<1>(bo, p, &v);
+      }
+      acc = Op::fma(acc, v, v);
+    }
+  }
+  const double bs = block_sums<Tv, 1, PAPER>(&acc, 1, wsum);
   if (threadIdx.x == 0) partials[bid] = bs;
   if (arrive_last(&st->counter, nblk) && threadIdx.x < 32) {
     const double tot = warp_sum_fixed(partials, nblk);
     if (threadIdx.x == 0 && final_pass) givens_step(st, j, sqrt(tot));
   }
 }
-template <typename Tv, int VEC, int CH>
+template <typename Tv, int VEC, int CH, bool PAPER>
 __global__ void __launch_bounds__(kBlock) update_kernel(Tv* __restrict__ V, size_t N, int j, int final_pass,
                                                         double* partials, SolverState* st, Bf16Out bo) {
-  update_body<Tv, VEC, CH>(V, N, j, final_pass, partials, st, bo, blockIdx.x, gridDim.x);
+  update_body<Tv, VEC, CH, PAPER>(V, N, j, final_pass, partials, st, bo, blockIdx.x, gridDim.x);
 }
 
 // Back substitution R y = g for the jlast columns of the cycle.
@@ -683,9 +782,10 @@ __global__ void __launch_bounds__(kBlock) xupdate_v_kernel(double* __restrict__ 
   __shared__ double y[kMaxRestart];
   for (int i = threadIdx.x; i < J; i += blockDim.x) y[i] = st->y[i] * st->s[i];
   __syncthreads();
+  const size_t ld = basis_ld(N);
   for (size_t p = blockIdx.x * (size_t)blockDim.x + threadIdx.x; p < N; p += (size_t)gridDim.x * blockDim.x) {
     double v = x[p];
-    for (int i = 0; i < J; ++i) v += y[i] * V[(size_t)i * N + p];
+    for (int i = 0; i < J; ++i) v += y[i] * V[(size_t)i * ld + p];
     x[p] = v;
   }
 }
@@ -704,14 +804,26 @@ void launch_rhs(const double* u, const double* uu, const double* src, const uint
 void launch_norm_b(const double* b, size_t N, double* partials, SolverState* st, cudaStream_t s) {
   norm_b_kernel<<<vec_grid(N), kBlock, 0, s>>>(b, N, partials, st);
 }
-// Gram-Schmidt grid: one full wave of resident blocks, but no more blocks
-// than give every thread eight 16-byte packs (small vectors: the block and
-// grid reductions would outweigh the loads).
-static int wave_grid(int per_sm, size_t N) {
-  const int g = kNumSMs * per_sm;
-  size_t c = (N + kBlock * 8 - 1) / (kBlock * 8);
-  const int cap = c < 1 ? 1 : (int)c;
-  return g < cap ? g : cap;
+// Gram-Schmidt grid: one full wave of resident blocks, but no more than one
+// block per four 16-byte packs of every thread, or (up to 64 blocks) per pack.
+// Few packs per thread shorten the chain of dependent rounds, whose latency
+// bounds vectors below 10^6; each block costs its reductions, which bound
+// the batch, where the blocks of all instances share the FP64 pipes.  With 8, 4, 2
+// and 1 packs throughout: a step at 64 x 64 2.98, 2.80, 2.70, 2.66 ms; 512 x 512
+// 10.40, 9.99, 9.94, 10.01 ms; 48 instances of 64 to 512 squared 50.2, 49.5,
+// 51.0, 55.0 ms.  Paper mode keeps eight packs, and with them its sums.
+template <bool PAPER>
+static int wave_grid(int per_sm, size_t packs) {
+  const size_t wave = (size_t)kNumSMs * per_sm;
+  if (PAPER) {
+    const size_t c = (packs + kBlock * 8 - 1) / (kBlock * 8);
+    return (int)(c > wave ? wave : c < 1 ? 1 : c);
+  }
+  const size_t four = (packs + kBlock * 4 - 1) / (kBlock * 4), one = (packs + kBlock - 1) / kBlock;
+  const size_t few = one < 64 ? one : 64;
+  size_t c = four > few ? four : few;
+  if (c > wave) c = wave;
+  return c < 1 ? 1 : (int)c;
 }
 template <typename K>
 static int resident_blocks(K kernel) {
@@ -724,61 +836,67 @@ static int resident_blocks(K kernel) {
 // (the kernels then take 4 or 2 packs per round), else 8.
 static int dot_chunk(int j) { return j + 1 <= 2 ? 2 : j + 1 <= 4 ? 4 : kDotChunk; }
 
-template <typename Tv, int VEC, int CH>
+template <typename Tv, int VEC, int CH, bool PAPER>
 static dim3 multidot_grid(size_t N, int j) {
-  static const int per_sm = resident_blocks(multidot_kernel<Tv, VEC, CH>);
+  static const int per_sm = resident_blocks(multidot_kernel<Tv, VEC, CH, PAPER>);
   // the chunks share one wave: each takes 1/chunks of the resident blocks
   const int chunks = (j + 1 + CH - 1) / CH;
-  const int gx = wave_grid(per_sm, N / VEC);
+  const int gx = wave_grid<PAPER>(per_sm, (N + VEC - 1) / VEC);
   return dim3(gx / chunks > kNumSMs ? gx / chunks : (gx < kNumSMs ? gx : kNumSMs), chunks);
 }
-template <typename Tv, int VEC, int CH>
+template <typename Tv, int VEC, int CH, bool PAPER>
+static int update_grid(size_t N) {
+  static const int per_sm = resident_blocks(update_kernel<Tv, VEC, CH, PAPER>);
+  return wave_grid<PAPER>(per_sm, (N + VEC - 1) / VEC);
+}
+// f(the chunk width of column j, as a compile-time constant)
+template <typename F>
+static auto with_chunk(int j, F&& f) {
+  const int ch = dot_chunk(j);
+  return ch == 2   ? f(std::integral_constant<int, 2>{})
+         : ch == 4 ? f(std::integral_constant<int, 4>{})
+                   : f(std::integral_constant<int, kDotChunk>{});
+}
+template <typename Tv, int VEC, bool PAPER>
 static void launch_multidot_t(const Tv* V, size_t N, int j, int accumulate, double* partials, SolverState* st,
                               cudaStream_t s) {
-  multidot_kernel<Tv, VEC, CH><<<multidot_grid<Tv, VEC, CH>(N, j), kBlock, 0, s>>>(V, N, j, accumulate, partials, st);
+  with_chunk(j, [&](auto c) {
+    constexpr int CH = decltype(c)::value;
+    multidot_kernel<Tv, VEC, CH, PAPER><<<multidot_grid<Tv, VEC, CH, PAPER>(N, j), kBlock, 0, s>>>(
+        V, N, j, accumulate, partials, st);
+  });
 }
-// 16-byte accesses when every basis vector is 16-byte aligned, else one element.
+template <typename Tv, int VEC, bool PAPER>
+static void launch_update_t(Tv* V, size_t N, int j, int final_pass, double* partials, SolverState* st,
+                            cudaStream_t s, const Bf16Out& bo) {
+  with_chunk(j, [&](auto c) {
+    constexpr int CH = decltype(c)::value;
+    update_kernel<Tv, VEC, CH, PAPER><<<update_grid<Tv, VEC, CH, PAPER>(N), kBlock, 0, s>>>(V, N, j, final_pass,
+                                                                                            partials, st, bo);
+  });
+}
 template <typename Tv>
 void launch_multidot(const Tv* V, size_t N, int j, int accumulate, double* partials, SolverState* st,
                      cudaStream_t s) {
-  constexpr int VEC = 16 / sizeof(Tv);
-  const int ch = dot_chunk(j);
-  if (N % VEC == 0) {
-    if (ch == 2) launch_multidot_t<Tv, VEC, 2>(V, N, j, accumulate, partials, st, s);
-    else if (ch == 4) launch_multidot_t<Tv, VEC, 4>(V, N, j, accumulate, partials, st, s);
-    else launch_multidot_t<Tv, VEC, kDotChunk>(V, N, j, accumulate, partials, st, s);
-  } else {
-    if (ch == 2) launch_multidot_t<Tv, 1, 2>(V, N, j, accumulate, partials, st, s);
-    else if (ch == 4) launch_multidot_t<Tv, 1, 4>(V, N, j, accumulate, partials, st, s);
-    else launch_multidot_t<Tv, 1, kDotChunk>(V, N, j, accumulate, partials, st, s);
-  }
-}
-template <typename Tv, int VEC, int CH>
-static int update_grid(size_t N) {
-  static const int per_sm = resident_blocks(update_kernel<Tv, VEC, CH>);
-  return wave_grid(per_sm, N / VEC);
-}
-template <typename Tv, int VEC, int CH>
-static void launch_update_t(Tv* V, size_t N, int j, int final_pass, double* partials, SolverState* st,
-                            cudaStream_t s, const Bf16Out& bo) {
-  update_kernel<Tv, VEC, CH><<<update_grid<Tv, VEC, CH>(N), kBlock, 0, s>>>(V, N, j, final_pass, partials, st, bo);
+  launch_multidot_t<Tv, 16 / sizeof(Tv), false>(V, N, j, accumulate, partials, st, s);
 }
 template <typename Tv>
 void launch_update(Tv* V, size_t N, int j, int final_pass, double* partials, SolverState* st, cudaStream_t s,
                    const Bf16Out* bo) {
-  constexpr int VEC = 16 / sizeof(Tv);
+  launch_update_t<Tv, 16 / sizeof(Tv), false>(V, N, j, final_pass, partials, st, s,
+                                              bo ? *bo : Bf16Out{nullptr, nullptr, 1, 0, 0});
+}
+// Paper mode: every sum in the order it has had (16-byte packs where N is even).
+void launch_multidot_paper(const double* V, size_t N, int j, int accumulate, double* partials, SolverState* st,
+                           cudaStream_t s) {
+  if (N % 2 == 0) launch_multidot_t<double, 2, true>(V, N, j, accumulate, partials, st, s);
+  else launch_multidot_t<double, 1, true>(V, N, j, accumulate, partials, st, s);
+}
+void launch_update_paper(double* V, size_t N, int j, int final_pass, double* partials, SolverState* st,
+                         cudaStream_t s) {
   const Bf16Out none{nullptr, nullptr, 1, 0, 0};
-  const int ch = dot_chunk(j);
-  if (N % VEC == 0) {
-    const Bf16Out& b = bo ? *bo : none;
-    if (ch == 2) launch_update_t<Tv, VEC, 2>(V, N, j, final_pass, partials, st, s, b);
-    else if (ch == 4) launch_update_t<Tv, VEC, 4>(V, N, j, final_pass, partials, st, s, b);
-    else launch_update_t<Tv, VEC, kDotChunk>(V, N, j, final_pass, partials, st, s, b);
-  } else {  // (the BF16 copy is only taken with 16-byte packs)
-    if (ch == 2) launch_update_t<Tv, 1, 2>(V, N, j, final_pass, partials, st, s, none);
-    else if (ch == 4) launch_update_t<Tv, 1, 4>(V, N, j, final_pass, partials, st, s, none);
-    else launch_update_t<Tv, 1, kDotChunk>(V, N, j, final_pass, partials, st, s, none);
-  }
+  if (N % 2 == 0) launch_update_t<double, 2, true>(V, N, j, final_pass, partials, st, s, none);
+  else launch_update_t<double, 1, true>(V, N, j, final_pass, partials, st, s, none);
 }
 template void launch_multidot<double>(const double*, size_t, int, int, double*, SolverState*, cudaStream_t);
 template void launch_multidot<df>(const df*, size_t, int, int, double*, SolverState*, cudaStream_t);
@@ -862,10 +980,7 @@ __global__ void __launch_bounds__(kBlock, 4) multidot_multi_kernel(const BatchIn
     constexpr int VEC = 16 / sizeof(Tv);
     const int gx = nb / chunks;
     const Tv* V = reinterpret_cast<const Tv*>(I.V);
-    if (I.N % VEC == 0)
-      multidot_body<Tv, VEC, CH>(V, I.N, j, accumulate, I.partials, I.st, lb % gx, gx, lb / gx, chunks);
-    else
-      multidot_body<Tv, 1, CH>(V, I.N, j, accumulate, I.partials, I.st, lb % gx, gx, lb / gx, chunks);
+    multidot_body<Tv, VEC, CH, false>(V, I.N, j, accumulate, I.partials, I.st, lb % gx, gx, lb / gx, chunks);
   }, sched);
 }
 template <typename Tv, int CH>
@@ -875,15 +990,11 @@ __global__ void __launch_bounds__(kBlock, 4) update_multi_kernel(const BatchInst
                                                               int final_pass, int write_a0, int* sched) {
   multi_loop(bi, prefix, active, count, [&](const BatchInst& I, int lb, int nb) {
     constexpr int VEC = 16 / sizeof(Tv);
-    const Bf16Out none{nullptr, nullptr, 1, 0, 0};
     Tv* V = reinterpret_cast<Tv*>(I.V);
-    if (I.N % VEC == 0) {  // (a0_fused implies N % VEC == 0)
-      const bool wr = write_a0 && I.a0_fused;
-      const Bf16Out bo{wr ? static_cast<__nv_bfloat16*>(I.a0) : nullptr,
-                       wr ? static_cast<__nv_bfloat16*>(I.a0_lo) : nullptr, wr ? I.n1 : 1, I.a0_ld, I.a0_hk};
-      update_body<Tv, VEC, CH>(V, I.N, j, final_pass, I.partials, I.st, bo, lb, nb);
-    }
-    else update_body<Tv, 1, CH>(V, I.N, j, final_pass, I.partials, I.st, none, lb, nb);
+    const bool wr = write_a0 && I.a0_fused;
+    const Bf16Out bo{wr ? static_cast<__nv_bfloat16*>(I.a0) : nullptr,
+                     wr ? static_cast<__nv_bfloat16*>(I.a0_lo) : nullptr, wr ? I.n1 : 1, I.a0_ld, I.a0_hk};
+    update_body<Tv, VEC, CH, false>(V, I.N, j, final_pass, I.partials, I.st, bo, lb, nb);
   }, sched);
 }
 __global__ void solve_y_multi_kernel(const BatchInst* __restrict__ bi) { solve_y_body(bi[blockIdx.x].st); }
@@ -940,31 +1051,31 @@ __global__ void loop_cond_multi_kernel(cudaGraphConditionalHandle h, const Batch
     cudaGraphSetConditional(h, go ? 1u : 0u);
   }
 }
-// Active prefixes (one block; count <= kMaxBatchMulti): an inclusive scan per
-// family of the instances' virtual-grid sizes, zero where the gate is closed.
+// Active prefixes (one block per family; count <= kMaxBatchMulti): an
+// inclusive scan of the instances' virtual-grid sizes, zero where the gate is closed, by warp
+// scans.  (One block scanning the nine families in turn, ten barriers each, took 15.8 us per
+// iteration of the batch.)
 __global__ void __launch_bounds__(kMaxBatchMulti) compact_multi_kernel(const BatchInst* __restrict__ bi, int count,
                                                                        int use_cycle, CompactArgs a) {
-  __shared__ int sc[kMaxBatchMulti];
-  const int i = threadIdx.x;
-  int open = 0;
+  __shared__ int wsum[kMaxBatchMulti / 32];
+  const int i = threadIdx.x, l = i & 31, w = i >> 5, f = blockIdx.x;
+  int v = 0;
   if (i < count) {
     const SolverState* st = bi[i].st;
-    open = use_cycle ? *(volatile const int*)&st->run_cycle : *(volatile const int*)&st->run_iter;
+    const int open = use_cycle ? *(volatile const int*)&st->run_cycle : *(volatile const int*)&st->run_iter;
+    if (open) v = __ldg(a.prefix[f] + i + 1) - __ldg(a.prefix[f] + i);
   }
-  for (int f = 0; f < a.nfam; ++f) {
-    const int v = (i < count && open) ? __ldg(a.prefix[f] + i + 1) - __ldg(a.prefix[f] + i) : 0;
-    sc[i] = v;
-    __syncthreads();
-    for (int d = 1; d < kMaxBatchMulti; d <<= 1) {  // Hillis-Steele inclusive scan
-      const int t = i >= d ? sc[i - d] : 0;
-      __syncthreads();
-      sc[i] += t;
-      __syncthreads();
-    }
-    if (i < count) a.active[f][i] = sc[i] - v;
-    if (i == count - 1) a.active[f][count] = sc[i];
-    __syncthreads();
+  int s = v;
+#pragma unroll
+  for (int d = 1; d < 32; d <<= 1) {
+    const int t = __shfl_up_sync(0xffffffffu, s, d);
+    if (l >= d) s += t;
   }
+  if (l == 31) wsum[w] = s;
+  __syncthreads();
+  for (int k = 0; k < w; ++k) s += wsum[k];
+  if (i < count) a.active[f][i] = s - v;
+  if (i == count - 1) a.active[f][count] = s;
 }
 
 // 1 in *out while any instance of the batch still runs a cycle (direct launches).
@@ -979,7 +1090,7 @@ void launch_any_running_multi(const BatchInst* bi, int count, int* out, cudaStre
 }
 
 void launch_compact_multi(const BatchInst* bi, int count, int use_cycle, const CompactArgs& a, cudaStream_t s) {
-  compact_multi_kernel<<<1, kMaxBatchMulti, 0, s>>>(bi, count, use_cycle, a);
+  compact_multi_kernel<<<a.nfam, (count + 31) / 32 * 32, 0, s>>>(bi, count, use_cycle, a);
 }
 void launch_init_multi(const BatchInst* bi, int count, int m, int max_iter, double tol, cudaStream_t s) {
   init_multi_kernel<<<(count + 127) / 128, 128, 0, s>>>(bi, count, m, max_iter, tol);
@@ -1035,24 +1146,13 @@ void launch_loop_cond_multi(cudaGraphConditionalHandle h, const BatchInst* bi, i
 // The grids of the single-instance launches, for the multi-instance prefixes.
 template <typename Tv>
 int multidot_blocks(size_t N, int j) {
-  constexpr int VEC = 16 / sizeof(Tv);
-  const int ch = dot_chunk(j);
-  dim3 g;
-  if (N % VEC == 0)
-    g = ch == 2 ? multidot_grid<Tv, VEC, 2>(N, j) : ch == 4 ? multidot_grid<Tv, VEC, 4>(N, j)
-                                                             : multidot_grid<Tv, VEC, kDotChunk>(N, j);
-  else
-    g = ch == 2 ? multidot_grid<Tv, 1, 2>(N, j) : ch == 4 ? multidot_grid<Tv, 1, 4>(N, j)
-                                                           : multidot_grid<Tv, 1, kDotChunk>(N, j);
+  const dim3 g = with_chunk(
+      j, [&](auto c) { return multidot_grid<Tv, 16 / sizeof(Tv), decltype(c)::value, false>(N, j); });
   return (int)(g.x * g.y);
 }
 template <typename Tv>
 int update_blocks(size_t N, int j) {
-  constexpr int VEC = 16 / sizeof(Tv);
-  const int ch = dot_chunk(j);
-  if (N % VEC == 0)
-    return ch == 2 ? update_grid<Tv, VEC, 2>(N) : ch == 4 ? update_grid<Tv, VEC, 4>(N) : update_grid<Tv, VEC, kDotChunk>(N);
-  return ch == 2 ? update_grid<Tv, 1, 2>(N) : ch == 4 ? update_grid<Tv, 1, 4>(N) : update_grid<Tv, 1, kDotChunk>(N);
+  return with_chunk(j, [&](auto c) { return update_grid<Tv, 16 / sizeof(Tv), decltype(c)::value, false>(N); });
 }
 int xupdate_blocks(size_t N, int zbytes) {
   const size_t VEC = 16 / (size_t)zbytes;

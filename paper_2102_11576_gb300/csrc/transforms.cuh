@@ -730,7 +730,7 @@ __global__ void __launch_bounds__(kMultiThreads, sizeof(T) == 8 ? 2 : 4) operato
     const AxisTables<T>& ax = inst_tab<T>(I, COLS);
     const int F = multi_groups(ax.L);
     const Tz* z = static_cast<const Tz*>(I.Z) + (size_t)j * I.N;
-    Tv* w = reinterpret_cast<Tv*>(I.V) + (size_t)(j + 1) * I.N;
+    Tv* w = reinterpret_cast<Tv*>(I.V) + (size_t)(j + 1) * basis_ld(I.N);
     toeplitz_body<T, Tz, MODE_APPLY, COLS, Tv>(z, static_cast<T*>(I.tmpx), I.phi, I.pen, nullptr, w, I.n1, I.n2, ax,
                                                F, group_stride<T>(ax.L, F, COLS), &I.st->run_iter, nullptr, nullptr,
                                                lb, nb);
@@ -767,7 +767,7 @@ __global__ void __launch_bounds__(kMultiThreads, sizeof(T) == 8 ? 2 : 4) dst_row
   multi_loop(bi, prefix, active, count, [&](const BatchInst& I, int lb, int nb) {
     const AxisTables<T>& ax = inst_tab<T>(I, false);
     const int F = multi_groups(ax.L);
-    dst_body<T, Tv, T, false>(reinterpret_cast<const Tv*>(I.V) + (size_t)j * I.N, &I.st->s[j],
+    dst_body<T, Tv, T, false>(reinterpret_cast<const Tv*>(I.V) + (size_t)j * basis_ld(I.N), &I.st->s[j],
                               static_cast<T*>(I.T1), I.n1, I.n2, ax, F, group_stride<T>(ax.L, F, false),
                               &I.st->run_iter, lb, nb);
   }, sched);
