@@ -84,6 +84,7 @@ struct DigitEpiParams {
   const void* z;       // DG_COLS: z (FP32 if z_float)
   int z_float;
   double pen;          // dt/eta
+  int early;           // trigger the next kernel of the chain at once (launch_digit)
   long long wait_cycles;
 };
 
@@ -216,7 +217,7 @@ __global__ void __launch_bounds__(kDgThreads, 1)
   }
   // everything above touches only this block; what the previous kernel wrote is read below
   pdl_wait();
-  pdl_trigger();
+  if (ep.early) pdl_trigger();
   if (gate && *(volatile const int*)gate == 0) return;
   if (warp == 0) {
     tmem_alloc(&tmem_base, kCols);
