@@ -454,6 +454,8 @@ void launch_finalize(double* x, size_t N, SolverState* st, cudaStream_t s);
 void launch_loop_cond(cudaGraphConditionalHandle h, SolverState* st, cudaStream_t s);
 void launch_restart_norm(const double* v, size_t N, double* partials, SolverState* st, const int* gate,
                          cudaStream_t s);
+void launch_residual_norm(const double* b, double* v, size_t N, double* partials, SolverState* st, const int* gate,
+                          cudaStream_t s);
 void launch_xupdate_v(double* x, const double* V, size_t N, SolverState* st, cudaStream_t s);
 void launch_adjoint_accum(const double* u_prev, const double* mu, const double* ax_u, const double* ay_u,
                           const uint8_t* phi, double dt, double ikx, double iky, double* lam_prev,

@@ -773,6 +773,27 @@ __global__ void __launch_bounds__(kBlock) restart_norm_kernel(const double* __re
   }
 }
 
+// V_0 = b - V_0 (V_0 holds M x), beta = ||V_0||, then the restart decision.  Memory-bound: 24 bytes
+// per element.
+__global__ void __launch_bounds__(kBlock) residual_norm_kernel(const double* __restrict__ b, double* __restrict__ v,
+                                                               size_t N, double* partials, SolverState* st,
+                                                               const int* gate) {
+  if (closed(gate)) return;
+  __shared__ double red[32];
+  double acc = 0.0;
+  for (size_t p = blockIdx.x * (size_t)blockDim.x + threadIdx.x; p < N; p += (size_t)gridDim.x * blockDim.x) {
+    const double r = b[p] - v[p];
+    v[p] = r;
+    acc += r * r;
+  }
+  const double bs = block_sum(acc, red);
+  if (threadIdx.x == 0) partials[blockIdx.x] = bs;
+  if (arrive_last(&st->counter, gridDim.x)) {
+    const double tot = sum_partials(partials, gridDim.x, red);
+    if (threadIdx.x == 0) restart_prep(st, sqrt(tot));
+  }
+}
+
 // x <- x + sum_i y_i v_i = x + sum_i (y_i s_i) V_i (left-preconditioned GMRES).
 __global__ void __launch_bounds__(kBlock) xupdate_v_kernel(double* __restrict__ x, const double* __restrict__ V,
                                                            size_t N, SolverState* st) {
@@ -925,6 +946,10 @@ void launch_adjoint_accum(const double* u_prev, const double* mu, const double* 
 void launch_restart_norm(const double* v, size_t N, double* partials, SolverState* st, const int* gate,
                          cudaStream_t s) {
   restart_norm_kernel<<<vec_grid(N), kBlock, 0, s>>>(v, N, partials, st, gate);
+}
+void launch_residual_norm(const double* b, double* v, size_t N, double* partials, SolverState* st, const int* gate,
+                          cudaStream_t s) {
+  residual_norm_kernel<<<vec_grid(N), kBlock, 0, s>>>(b, v, N, partials, st, gate);
 }
 void launch_xupdate_v(double* x, const double* V, size_t N, SolverState* st, cudaStream_t s) {
   xupdate_v_kernel<<<vec_grid(N), kBlock, 0, s>>>(x, V, N, st);
