@@ -124,9 +124,6 @@ __device__ __forceinline__ void tma_load_3d(void* dst, const CUtensorMap* map, i
       "l"((uint64_t)map), "r"(x), "r"(y), "r"(z), "r"(smem_u32(bar))
       : "memory");
 }
-__device__ __forceinline__ void mbar_arrive(uint64_t* bar) {
-  asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(bar)) : "memory");
-}
 // 32 lanes x 2 columns of tensor memory (no wait)
 __device__ __forceinline__ void tmem_ld2_nowait(uint32_t taddr, uint32_t* r) {
   asm volatile("tcgen05.ld.sync.aligned.32x32b.x2.b32 {%0, %1}, [%2];" : "=r"(r[0]), "=r"(r[1]) : "r"(taddr));
@@ -183,10 +180,12 @@ __device__ __forceinline__ uint32_t dg_exponent(double x) {
 // that leave SMs idle (dg_bn).
 //
 // Roles: warp 0 lane 0 loads (A in a ring of six slots, S double-buffered),
-// warps 1 and 2 issue the MMAs of groups 0..3 and 4..7; step[i] counts the
-// products with A_i done.  As the ring has six slots, A_i of the next slice is
+// warps 1 and 2 issue the MMAs of groups 0..3 and 4..7; step[i] counts both
+// warps' products with A_i done (the top warp has none for i >= 4 and just
+// arrives, once it has seen A_i land).  As the ring has six slots, A_i of the next slice is
 // loaded after step i + 2 of this one (i < 6) or step i - 6 of the next: no
-// step can complete twice before the loader's wait has seen it, so the waits'
+// step can complete twice before the loader's wait has seen it, and no slot
+// is refilled before both issuing warps have seen what it held, so the waits'
 // phase parities are never ambiguous.  All sixteen warps add up and store.
 template <int EPI, int BN>
 __global__ void __launch_bounds__(kDgThreads, 1)
@@ -207,7 +206,7 @@ __global__ void __launch_bounds__(kDgThreads, 1)
   const int warp = __shfl_sync(0xffffffffu, (int)(threadIdx.x >> 5), 0), lane = threadIdx.x & 31;
   if (threadIdx.x == 0) {
     for (int s = 0; s < kDgASlots; ++s) mbar_init(&fullA[s], 1);
-    for (int s = 0; s < kDgDigits; ++s) mbar_init(&step[s], s < 4 ? 2 : 1);  // groups 0..3 end with A_3
+    for (int s = 0; s < kDgDigits; ++s) mbar_init(&step[s], 2);
     for (int s = 0; s < 2; ++s) {
       mbar_init(&fullB[s], 1);
       mbar_init(&done[s], 2);
@@ -298,7 +297,10 @@ __global__ void __launch_bounds__(kDgThreads, 1)
             stop = true;
             break;
           }
-          if (top && i >= 4) continue;  // (waited for: every phase of every slot is seen in turn)
+          if (top && i >= 4) {  // groups 0..3 end with A_3
+            mbar_arrive(&step[i]);
+            continue;
+          }
           tc_fence_after();
           // groups s0 .. s0 + cnt - 1 from the digits s0 - i .. of S
           const int s0 = top ? i : (i < 4 ? 4 : i), cnt = top ? 4 - i : (i < 4 ? 4 : 8 - i);
