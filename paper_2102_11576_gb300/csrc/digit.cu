@@ -747,7 +747,9 @@ template <typename Tin, int CPB>
 static void launch_fold(DigitOperator* p, const Tin* z, double* pre, const int* gate, cudaStream_t s) {
   const int n1 = p->n1, n2 = p->n2, rblocks = fold_rblocks(n1, n2), smem = CPB * (n2 + 1) * (int)sizeof(double);
   auto k = digit_fold_kernel<Tin, CPB>;
-  if (smem > 48 * 1024) cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+  // (always, and always the largest: the limit is the function's, for every context, and the
+  // kernel's static shared memory counts towards the 48 KB that need none)
+  cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, CPB * (kDgMaxN + 1) * (int)sizeof(double));
   launch_pdl(k, dim3(fold_blocks(n1, n2)), dim3(256), smem, s, z, n1, n2, rblocks,
              (const double*)p->near, pre, p->R.d, p->R.plane(), p->R.hk, p->exps, p->C.d, p->C.plane(), p->C.hk,
              p->exps + n2, p->err, gate);

@@ -1,0 +1,47 @@
+"""The FP64 forms' digit products on what test_gpu_digit.py does not reach."""
+import numpy as np
+import pytest
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+if not torch.cuda.is_available():
+    pytest.skip("no CUDA device", allow_module_level=True)
+
+from paper_2102_11576_gb300 import workloads  # noqa: E402
+from test_gpu_digit import solver  # noqa: E402
+
+
+def few_rows(w, count=8):
+    """A field that is zero but for `count` rows, the first and the last among them, and those rows."""
+    rows = np.unique(np.linspace(0, w["n2"] - 1, count).astype(int))
+    z = np.zeros_like(w["field"])
+    z[rows] = w["field"][rows]
+    return z, rows
+
+
+def operator_error(s, w, got, z, rows):
+    """|got - M z| over and outside Omega and its bound there, in units of |z| (2-norm): M's middle
+    diagonals in FP64, six roundings of at most 2^-53 of the coefficients' sum, and
+    two products of the rest: 8 * 2^-53 of that sum."""
+    t, pen = s.tables(), np.longdouble(s.params()["pen"])
+    tx, ty = t["t_x"].astype(np.longdouble), t["t_y"].astype(np.longdouble)
+    zl, ref, out = z[rows].astype(np.longdouble), z.astype(np.longdouble), w["in_omega"] == 0
+    n1, n2 = w["n1"], w["n2"]
+    ref[rows] -= zl @ tx[np.abs(np.subtract.outer(np.arange(n1), np.arange(n1)))]
+    ref -= ty[np.abs(np.subtract.outer(np.arange(n2), rows))] @ zl
+    ref += pen * out * z
+    err, norm = got - ref, np.sqrt((z.astype(np.longdouble) ** 2).sum())
+    scale = 1 + 2 * (np.abs(tx).sum() + np.abs(ty).sum())
+    return [(np.sqrt((err[sel] ** 2).sum()), 8 * 2.0 ** -53 * c * norm) for sel, c in ((~out, scale), (out, scale + pen))]
+
+
+# four columns of the fold in shared memory: 48 KB, or less by up to the kernel's static 1 KB
+@pytest.mark.parametrize("n1,n2", [(608, 1503), (608, 1504), (609, 1535), (608, 1536)])
+def test_operator_near_the_plain_limit_of_shared_memory(n1, n2):
+    w = workloads.random_problem(70, n1, n2)
+    z, rows = few_rows(w)
+    s = solver(w)
+    for err, bound in operator_error(s, w, s.apply_M(torch.as_tensor(z).cuda()).cpu().numpy(), z, rows):
+        assert err <= bound
+    s.close()
