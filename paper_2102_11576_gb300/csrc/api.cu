@@ -278,7 +278,7 @@ int cuda_fail(cudaError_t e) {
 
 int check_launch(rsfde_ctx* c) {
   if (take_unsupported_launch()) return RSFDE_EINVAL;
-  return cuda_fail(cudaGetLastError());
+  return cuda_fail(take_launch_error());
 }
 
 cudaEvent_t prof_event(rsfde_ctx* c) {
@@ -426,7 +426,7 @@ int ensure_digit_operator(rsfde_ctx* c) {
   if (c->dop || c->opts.matvec_prec != RSFDE_FP64 || left_variant(c) || !digit_sizes_ok(c->n1, c->n2)) return RSFDE_OK;
   if (digit_operator_create(&c->dop, c->n1, c->n2, c->stream) != RSFDE_OK) return RSFDE_OK;
   if (!digit_operator_params(c->dop, c->hx_axis.t, c->hy_axis.t, c->stream)) {
-    cudaGetLastError();
+    take_launch_error();
     digit_operator_destroy(c->dop);
     c->dop = nullptr;
     return RSFDE_OK;
@@ -847,7 +847,7 @@ int build_cycle_graph(rsfde_ctx* c) {
   c->prof_on = prof;
   if (e == cudaSuccess) e = cudaGraphInstantiate(&c->graph_exec, c->graph, 0);
   if (e != cudaSuccess) {
-    cudaGetLastError();
+    take_launch_error();
     return cuda_fail(e);
   }
   c->graph_key = graph_key(c);
@@ -1543,7 +1543,7 @@ int build_batch_graph_multi(rsfde_batch* b, int later) {
   if (e == cudaSuccess) e = cudaGraphInstantiate(&b->exec[later], g, 0);
   cudaGraphDestroy(g);
   if (e != cudaSuccess) {
-    cudaGetLastError();
+    take_launch_error();
     return cuda_fail(e);
   }
   // launches: 5 in the prologue (reset, right sides, compaction, residual
@@ -1578,7 +1578,7 @@ int run_batch_step_direct(rsfde_batch* b, int later) {
     b->launches += b->launches_per_body;  // the body, its loop check counted as the condition kernel
   }
   launch_finish_rotate_multi(b->inst, b->g_fin, s);
-  return cuda_fail(cudaGetLastError());
+  return cuda_fail(take_launch_error());
 }
 
 // Builds the graph of one time step of every instance: per instance the
@@ -1624,7 +1624,7 @@ int build_batch_graph(rsfde_batch* b, int later) {
   if (e == cudaSuccess) e = cudaGraphInstantiate(&b->exec[later], g, 0);
   cudaGraphDestroy(g);
   if (e != cudaSuccess) {
-    cudaGetLastError();
+    take_launch_error();
     return cuda_fail(e);
   }
   return RSFDE_OK;

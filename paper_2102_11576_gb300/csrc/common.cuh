@@ -35,7 +35,7 @@ inline void launch_pdl(void (*k)(KArgs...), dim3 grid, dim3 block, size_t smem, 
   attr[0].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
-  cudaLaunchKernelEx(&cfg, k, args...);  // errors surface through cudaGetLastError
+  cudaLaunchKernelEx(&cfg, k, args...);  // errors surface through take_launch_error
 }
 constexpr int kBlock = 256;      // threads per block of the grid-vector kernels
 

@@ -444,7 +444,7 @@ int digit_plan_create(DigitPlan** out, int n1, int n2, cudaStream_t s) {
   const size_t se = ((size_t)nexp * sizeof(int) + 255) / 256 * 256;
   const size_t stab = (size_t)2 * (kDgMaxN + 1) * sizeof(long long);
   if (cudaMalloc(&p->mem, sx + sy + sw + si + se + 256 + stab) != cudaSuccess) {
-    cudaGetLastError();
+    take_launch_error();
     delete p;
     return RSFDE_ENOMEM;
   }
@@ -465,7 +465,7 @@ int digit_plan_create(DigitPlan** out, int n1, int n2, cudaStream_t s) {
   for (DigitMat* m : {&p->Sx, &p->Sy})
     for (int k = 0; k < 3; ++k) good = good && digit_map(m, &m->map[k], 64 >> k, kDgDigits);
   if (!good) {
-    cudaGetLastError();
+    take_launch_error();
     digit_plan_destroy(p);
     return RSFDE_ECUDA;
   }
@@ -534,7 +534,7 @@ template <int EPI, int BN>
 static void launch_digit_bn(const DigitMat& A, const DigitMat& S, const DigitEpiParams& ep, int* err, const int* gate,
                             cudaStream_t s) {
   auto k = digit_gemm_kernel<EPI, BN>;
-  cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, dg_smem(BN));
+  raise_smem_limit((const void*)k, dg_smem(BN));
   launch_pdl(k, dim3((ep.N + BN - 1) / BN, (ep.M + kDgBM - 1) / kDgBM), dim3(kDgThreads), dg_smem(BN), s, A.map[0],
              S.map[BN == 64 ? 0 : BN == 32 ? 1 : 2], ep, err, gate);
 }
@@ -709,7 +709,7 @@ int digit_operator_create(DigitOperator** out, int n1, int n2, cudaStream_t s) {
   }
   const size_t se = ((size_t)(n1 + n2) * sizeof(int) + 255) / 256 * 256;
   if (cudaMalloc(&p->mem, off[4] + se + 256 + kDgMaxN * sizeof(long long)) != cudaSuccess) {
-    cudaGetLastError();
+    take_launch_error();
     delete p;
     return RSFDE_ENOMEM;
   }
@@ -725,7 +725,7 @@ int digit_operator_create(DigitOperator** out, int n1, int n2, cudaStream_t s) {
   for (DigitMat* m : {&p->R, &p->Ty})
     for (int k = 0; k < 3; ++k) good = good && digit_map(m, &m->map[k], 64 >> k, kDgDigits);
   if (!good) {
-    cudaGetLastError();
+    take_launch_error();
     digit_operator_destroy(p);
     return RSFDE_ECUDA;
   }
@@ -749,7 +749,7 @@ static void launch_fold(DigitOperator* p, const Tin* z, double* pre, const int* 
   auto k = digit_fold_kernel<Tin, CPB>;
   // (always, and always the largest: the limit is the function's, for every context, and the
   // kernel's static shared memory counts towards the 48 KB that need none)
-  cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, CPB * (kDgMaxN + 1) * (int)sizeof(double));
+  raise_smem_limit((const void*)k, CPB * (kDgMaxN + 1) * (int)sizeof(double));
   launch_pdl(k, dim3(fold_blocks(n1, n2)), dim3(256), smem, s, z, n1, n2, rblocks,
              (const double*)p->near, pre, p->R.d, p->R.plane(), p->R.hk, p->exps, p->C.d, p->C.plane(), p->C.hk,
              p->exps + n2, p->err, gate);

@@ -297,14 +297,14 @@ static void launch_gemm_t(const Bf16Mat& A, const Bf16Mat& B, int M, int N, int 
   if constexpr (NT == 3) {
     if (tiles > kNumSMs && tiles <= 2L * kNumSMs) {
       auto k = dst_gemm_kernel<EPI, NT, SYM, BN, 2>;
-      cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+      raise_smem_limit((const void*)k, smem);
       launch_pdl(k, dim3(kNumSMs), dim3(gemm_threads(NT)), smem, s, A.map_hi, A.map_lo, bh, bl, K, ep, err,
                  gate);
       return;
     }
   }
   auto k = dst_gemm_kernel<EPI, NT, SYM, BN, 1>;
-  cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+  raise_smem_limit((const void*)k, smem);
   launch_pdl(k, dim3(gx, gy, channels), dim3(gemm_threads(NT)), smem, s, A.map_hi, A.map_lo, bh, bl, K, ep, err,
              gate);
 }
@@ -402,7 +402,7 @@ bool bf16_plan_a0(const Bf16Plan* p, int vec, Bf16Out* out) {
 }
 
 template <typename Tz, typename Tin>
-int bf16_precond(Bf16Plan* p, const Tin* v, const double* vscale, Tz* z, const uint8_t* phi, double pen,
+void bf16_precond(Bf16Plan* p, const Tin* v, const double* vscale, Tz* z, const uint8_t* phi, double pen,
                  const int* gate, cudaStream_t s, bool skip_split, const double* zscale, cudaEvent_t* ev) {
   const int n1 = p->n1, n2 = p->n2;
   if (skip_split) {
@@ -427,7 +427,6 @@ int bf16_precond(Bf16Plan* p, const Tin* v, const double* vscale, Tz* z, const u
     else launch_gemm<EPI_SPLIT_T>(p, k, g.hk, *g.A, *g.B, g.M, g.n, g.channels, g.ep, gate, s);
     if (ev) cudaEventRecord(ev[k + 1], s);
   }
-  return cudaGetLastError() == cudaSuccess ? RSFDE_OK : RSFDE_ECUDA;
 }
 
 // Times the chain with every GEMM 64 wide, then 128 wide (reps applications
@@ -533,7 +532,7 @@ static void launch_group_t(const GemmGroupDesc* d, int count, const int* active,
                            cudaStream_t s) {
   auto k = dst_gemm_group_kernel<EPI, 3, 64>;
   constexpr int smem = gemm_group_smem(3, 64);
-  cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+  raise_smem_limit((const void*)k, smem);
   k<<<max_tiles, kGroupThreads, smem, s>>>(d, active, count, j, err);
 }
 static_assert(kGroupMaxInstances == kMaxBatchMulti, "the grouped GEMMs stage the batch's whole prefix");
@@ -580,22 +579,22 @@ void launch_split_multi(const BatchInst* bi, const MultiGrid& g, int j, cudaStre
   split_multi_kernel<<<g.total < grid ? g.total : grid, kBlock, 0, s>>>(bi, g.prefix, g.active, g.count, j);
 }
 
-template int bf16_precond<float, double>(Bf16Plan*, const double*, const double*, float*, const uint8_t*, double,
+template void bf16_precond<float, double>(Bf16Plan*, const double*, const double*, float*, const uint8_t*, double,
                                          const int*, cudaStream_t, bool, const double*,
                                          cudaEvent_t*);
-template int bf16_precond<double, double>(Bf16Plan*, const double*, const double*, double*, const uint8_t*,
+template void bf16_precond<double, double>(Bf16Plan*, const double*, const double*, double*, const uint8_t*,
                                           double, const int*, cudaStream_t, bool, const double*,
                                          cudaEvent_t*);
-template int bf16_precond<float, df>(Bf16Plan*, const df*, const double*, float*, const uint8_t*, double,
+template void bf16_precond<float, df>(Bf16Plan*, const df*, const double*, float*, const uint8_t*, double,
                                      const int*, cudaStream_t, bool, const double*,
                                          cudaEvent_t*);
-template int bf16_precond<double, df>(Bf16Plan*, const df*, const double*, double*, const uint8_t*, double,
+template void bf16_precond<double, df>(Bf16Plan*, const df*, const double*, double*, const uint8_t*, double,
                                       const int*, cudaStream_t, bool, const double*,
                                          cudaEvent_t*);
-template int bf16_precond<float, float>(Bf16Plan*, const float*, const double*, float*, const uint8_t*, double,
+template void bf16_precond<float, float>(Bf16Plan*, const float*, const double*, float*, const uint8_t*, double,
                                         const int*, cudaStream_t, bool, const double*,
                                          cudaEvent_t*);
-template int bf16_precond<double, float>(Bf16Plan*, const float*, const double*, double*, const uint8_t*, double,
+template void bf16_precond<double, float>(Bf16Plan*, const float*, const double*, double*, const uint8_t*, double,
                                          const int*, cudaStream_t, bool, const double*,
                                          cudaEvent_t*);
 

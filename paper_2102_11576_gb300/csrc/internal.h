@@ -117,6 +117,12 @@ int max_groups(int L, int items);
 // nothing and raises a flag that the next launch check reports.
 void note_unsupported_launch();
 bool take_unsupported_launch();
+// Raises a kernel's limit of dynamic shared memory.  A successful
+// cudaFuncSetAttribute clears the runtime's last error, so a refused launch before it is
+// kept here (per thread, as the runtime's is), for take_launch_error: the
+// first error since the last call of it.
+void raise_smem_limit(const void* kernel, int bytes);
+cudaError_t take_launch_error();
 // tmpx: scratch of N values of the arithmetic type T between the passes:
 // z - A_x z + pen phi z when phi is given, else A_x z
 template <typename T, typename Tin>
@@ -185,8 +191,9 @@ void bf16_plan_set_wait(Bf16Plan* p, long long cycles);  // <= 0: the default bo
 // skip_split: the first operand was already written (update_kernel's Bf16Out,
 // unscaled), and zscale multiplies the result instead.
 // ev: if set, five events recorded before the first GEMM and after each (timing).
+// A launch's error is left for take_launch_error.
 template <typename Tz, typename Tin>
-int bf16_precond(Bf16Plan* p, const Tin* v, const double* vscale, Tz* z, const uint8_t* phi, double pen,
+void bf16_precond(Bf16Plan* p, const Tin* v, const double* vscale, Tz* z, const uint8_t* phi, double pen,
                  const int* gate, cudaStream_t s, bool skip_split = false, const double* zscale = nullptr,
                  cudaEvent_t* ev = nullptr);
 // Measured tile width (64 or 128) per GEMM of the chain, recorded in the plan.

@@ -159,5 +159,5 @@ extern "C" int rsfde_dst2_noalloc(int32_t n1, int32_t n2, const double* v, doubl
   const AxisTables<double> ty = device_axis(s_tables_addr[dev], 1, n2, L2, lg2);
   launch_dst_rows<double, double>(v, nullptr, s_scratch_addr[dev], n1, n2, tx, nullptr, s);
   launch_dst_cols<double, double, double>(s_scratch_addr[dev], out, n1, n2, ty, s);
-  return cudaGetLastError() == cudaSuccess ? RSFDE_OK : RSFDE_ECUDA;
+  return take_launch_error() == cudaSuccess ? RSFDE_OK : RSFDE_ECUDA;
 }

@@ -1,6 +1,7 @@
 // transforms.cu -- process-wide state of the transform launchers: the
 // tile-shape table the autotuner records, the shape it forces while timing,
-// and the flag of a launch with no kernel for its (type, mode) pair.  The
+// the flag of a launch with no kernel for its (type, mode) pair, and a
+// launch's error until it is reported.  The
 // kernels and launchers are in transforms.cuh, instantiated per arithmetic
 // type in transforms_f64.cu, transforms_f32.cu and transforms_df_a.cu, _b.cu and _c.cu.
 #include <atomic>
@@ -12,6 +13,7 @@ namespace rsfde {
 static int g_tuned[TK_COUNT][16][2];
 static thread_local int g_force_groups = 0;
 static std::atomic<int> g_unsupported{0};
+static thread_local cudaError_t g_launch_error = cudaSuccess;
 
 void tune_force_groups(int F) { g_force_groups = F; }
 int tune_forced() { return g_force_groups; }
@@ -23,6 +25,21 @@ int tune_lookup(int kind, int log2L, int wide) {
 }
 void note_unsupported_launch() { g_unsupported.store(1); }
 bool take_unsupported_launch() { return g_unsupported.exchange(0) != 0; }
+static void keep_launch_error() {
+  const cudaError_t e = cudaGetLastError();
+  if (g_launch_error == cudaSuccess) g_launch_error = e;
+}
+void raise_smem_limit(const void* kernel, int bytes) {
+  keep_launch_error();
+  cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+  keep_launch_error();
+}
+cudaError_t take_launch_error() {
+  keep_launch_error();
+  const cudaError_t e = g_launch_error;
+  g_launch_error = cudaSuccess;
+  return e;
+}
 
 template int max_groups<double>(int, int);
 template int max_groups<float>(int, int);
