@@ -91,7 +91,7 @@ std::vector<uint2> build_exact_tables(const std::vector<double>& t, int L, int* 
 
 template <typename K>
 static void exact_smem(K kernel, size_t bytes) {
-  if (bytes > 48 * 1024) raise_smem_limit((const void*)kernel, (int)bytes);
+  if (bytes > kPlainSmem) raise_smem_limit((const void*)kernel, (int)bytes);
 }
 
 // The transform kernel for rows or columns: blockIdx.y is the prime.

@@ -122,6 +122,9 @@ bool take_unsupported_launch();
 // kept here (per thread, as the runtime's is), for take_launch_error: the
 // first error since the last call of it.
 void raise_smem_limit(const void* kernel, int bytes);
+// Dynamic bytes that need no raised limit: 48 KB less what the kernels hold statically (about
+// 5 KB at most, the batch's active prefix), which counts towards it.
+constexpr size_t kPlainSmem = 40 * 1024;
 cudaError_t take_launch_error();
 // tmpx: scratch of N values of the arithmetic type T between the passes:
 // z - A_x z + pen phi z when phi is given, else A_x z

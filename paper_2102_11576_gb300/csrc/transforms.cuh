@@ -585,7 +585,7 @@ static size_t group_smem(int L, int F, bool cols) {
 
 template <typename K>
 static void set_smem(K kernel, size_t bytes) {
-  if (bytes > 48 * 1024) raise_smem_limit((const void*)kernel, (int)bytes);
+  if (bytes > kPlainSmem) raise_smem_limit((const void*)kernel, (int)bytes);
 }
 
 // phi != nullptr: tmpx = z - A_x z + pen phi z (ahead of a MODE_APPLY,
