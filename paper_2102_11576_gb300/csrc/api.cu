@@ -333,6 +333,8 @@ void prof_harvest(rsfde_ctx* c) {
 }
 
 int build_tables(rsfde_ctx* c) {
+  const double pen0 = c->pen;
+  const int xst0 = c->xex.tab.St, yst0 = c->yex.tab.St;
   c->hx = (c->bx - c->ax) / (c->n1 + 1);  // Section 2
   c->hy = (c->by - c->ay) / (c->n2 + 1);
   c->cx = c->dt * c->kx * riesz_c(c->alpha1) / std::pow(c->hx, c->alpha1);
@@ -355,6 +357,9 @@ int build_tables(rsfde_ctx* c) {
     c->dop = nullptr;
     c->graph_key = -1;
   }
+  // dt/eta and the scales of the exact products are arguments of captured launches (the
+  // other parameters' tables are read where they lie)
+  if (c->pen != pen0 || c->xex.tab.St != xst0 || c->yex.tab.St != yst0) c->graph_key = -1;
   return RSFDE_OK;
 }
 

@@ -1,0 +1,40 @@
+"""New parameters after a solve whose cycle was captured: the next solve is that of a
+solver made with them, bit for bit (the same launches on the same values)."""
+import pytest
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+if not torch.cuda.is_available():
+    pytest.skip("no CUDA device", allow_module_level=True)
+
+from paper_2102_11576_gb300 import Solver, workloads  # noqa: E402
+
+FORMS = {
+    "fp64": dict(),
+    "mixed": dict(precond="bf16x3", matvec="fp32", basis="fp64", resid="exact"),
+    "fp32": dict(precond="fp32", matvec="fp32", basis="fp64", resid="exact"),
+    "df32": dict(precond="fp32", matvec="df32", basis="df32", resid="fp64"),
+    "paper": dict(variant="gmres_left", tol=1e-8),
+}
+
+
+def solver(w, **kw):
+    return Solver(w["n1"], w["n2"], w["box"], w["in_omega"], w["alpha1"], w["alpha2"], w["kx"], w["ky"], w["dt"],
+                  w["eta"], **kw)
+
+
+# dt moves dt/eta; kx and ky move the powers of two that scale the exact products
+@pytest.mark.parametrize("kx,ky,dt", [(1.0, 1.0, 7.0), (40.0, 0.02, 1.0), (0.3, 5.0, 0.2)])
+@pytest.mark.parametrize("form", list(FORMS))
+def test_solve_after_new_parameters(form, kx, ky, dt):
+    w = dict(workloads.random_problem(90, 75, 52), eta=1e-4)
+    b = torch.as_tensor(w["field"]).cuda()
+    new = dict(w, kx=kx * w["kx"], ky=ky * w["ky"], dt=dt * w["dt"])
+    s, fresh = solver(w, **FORMS[form]), solver(new, **FORMS[form])
+    s.solve(b)
+    s.set_params(new["kx"], new["ky"], new["dt"])
+    (x, st), (ref, st_ref) = s.solve(b), fresh.solve(b)
+    assert torch.equal(x, ref) and st["iters"] == st_ref["iters"]
+    s.close()
+    fresh.close()
