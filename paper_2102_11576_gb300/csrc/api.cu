@@ -1967,6 +1967,7 @@ int64_t rsfde_kernel_launches(const rsfde_ctx* c) { return c ? c->launches : 0; 
 
 int rsfde_set_wait_cycles(rsfde_ctx* c, int64_t cycles) {
   if (!c || cycles < 0) return RSFDE_EINVAL;
+  if (cycles != c->wait_cycles) c->graph_key = -1;  // captured launches carry the old bound
   c->wait_cycles = cycles;
   bf16_plan_set_wait(c->bf16, cycles);
   digit_plan_set_wait(c->digit, cycles);

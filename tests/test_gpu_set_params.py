@@ -8,7 +8,7 @@ pytestmark = pytest.mark.gpu
 if not torch.cuda.is_available():
     pytest.skip("no CUDA device", allow_module_level=True)
 
-from paper_2102_11576_gb300 import Solver, workloads  # noqa: E402
+from paper_2102_11576_gb300 import RsfdeError, Solver, workloads  # noqa: E402
 
 FORMS = {
     "fp64": dict(),
@@ -38,3 +38,18 @@ def test_solve_after_new_parameters(form, kx, ky, dt):
     assert torch.equal(x, ref) and st["iters"] == st_ref["iters"]
     s.close()
     fresh.close()
+
+
+@pytest.mark.parametrize("form", ["fp64", "mixed"])
+def test_a_new_wait_bound_holds_in_a_captured_solve(form):
+    w = dict(workloads.random_problem(91, 150, 90), eta=1e-4)
+    b = torch.as_tensor(w["field"]).cuda()
+    s = solver(w, **FORMS[form])
+    x = s.solve(b)[0].clone()
+    s.set_wait_cycles(1)
+    with pytest.raises(RsfdeError) as e:
+        s.solve(b)
+    assert e.value.name == "ETIMEOUT"
+    s.set_wait_cycles(0)
+    assert torch.equal(s.solve(b)[0], x)
+    s.close()
