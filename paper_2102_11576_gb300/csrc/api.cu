@@ -410,6 +410,7 @@ int ensure_bf16(rsfde_ctx* c) {
     cudaStreamSynchronize(c->stream);
     bf16_plan_destroy(c->bf16);
     c->bf16 = nullptr;
+    c->graph_key = -1;  // captured launches point into the old plan
   }
   const int rc = bf16_plan_create(&c->bf16, c->n1, c->n2, nt, c->x32.tab.lam, c->y32.tab.lam, c->phi, c->stream);
   if (rc == RSFDE_OK) bf16_plan_set_wait(c->bf16, c->wait_cycles);

@@ -53,3 +53,16 @@ def test_a_new_wait_bound_holds_in_a_captured_solve(form):
     s.set_wait_cycles(0)
     assert torch.equal(s.solve(b)[0], x)
     s.close()
+
+
+def test_changing_the_preconditioner_and_back_rebuilds_what_was_captured():
+    w = dict(workloads.random_problem(92, 150, 90), eta=1e-4)
+    b = torch.as_tensor(w["field"]).cuda()
+    s = solver(w, **FORMS["mixed"])
+    x = s.solve(b)[0].clone()
+    s.set_options(precond="bf16")  # frees the split-BF16 plan
+    held = torch.empty(1 << 26, dtype=torch.uint8, device="cuda")
+    s.set_options(precond="bf16x3")
+    assert torch.equal(s.solve(b)[0], x)
+    del held
+    s.close()
