@@ -450,7 +450,7 @@ __global__ void __launch_bounds__(kDgThreads, 1)
           double* __restrict__ out = static_cast<double*>(ep.out0);
           const size_t o = (size_t)nn * ep.ldo + mm;
           if constexpr (EPI == DG_COLS) {
-            if (mvalid) {
+            if (mvalid && !(mir && nn == n)) {  // (the middle once: out may be z itself)
               double v = pre[q][mir] - ldexp_i64(w, kx);
               if (phi[q][mir])
                 v = __fma_rn(ep.pen,

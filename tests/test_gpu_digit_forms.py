@@ -45,3 +45,14 @@ def test_operator_near_the_plain_limit_of_shared_memory(n1, n2):
     for err, bound in operator_error(s, w, s.apply_M(torch.as_tensor(z).cuda()).cpu().numpy(), z, rows):
         assert err <= bound
     s.close()
+
+
+@pytest.mark.parametrize("n1,n2", [(1, 1), (33, 31), (64, 65), (70, 129)])
+def test_operators_in_place(n1, n2):
+    w = workloads.random_problem(71, n1, n2)
+    s = solver(w)
+    v = torch.as_tensor(w["field"]).cuda()
+    for op in (s.apply_M, s.apply_precond, s.dst2):
+        ref, x = op(v), v.clone()
+        assert torch.equal(op(x, out=x), ref)
+    s.close()
