@@ -243,8 +243,9 @@ int rsfde_batch_create(rsfde_batch** out, int32_t count, const rsfde_grid* grids
 int rsfde_batch_set(rsfde_batch* b, int32_t i, const double* u0, const double* src);
 /* Advances every instance by `steps` implicit steps (f = u - u^3 + src, Eq. 2.17).
  * stats: HOST array of `count` (statistics of each instance's last step) or
- * NULL.  Returns RSFDE_ETIMEOUT if a grouped split-BF16 GEMM's pipeline wait
- * gave up (its output was incomplete; the batch stays usable), else the first
+ * NULL.  Returns RSFDE_ETIMEOUT if a pipeline wait of the split-BF16 GEMMs or
+ * of an instance's FP64 digit products gave up in any of the steps (what it left
+ * was incomplete: set the instances anew; the batch stays usable), else the first
  * non-OK instance status, else RSFDE_OK.  Synchronises. */
 int rsfde_batch_run(rsfde_batch* b, int32_t steps, rsfde_stats* stats);
 /* Copies instance i's current u^k to the device array u_out (N_i doubles). */
@@ -253,6 +254,10 @@ int64_t rsfde_batch_kernel_launches(rsfde_batch* b);
 void rsfde_batch_destroy(rsfde_batch* b);
 
 /* ---- operator-level entry points (each one step of the hot path) --------- */
+/* These calls only enqueue work (the split-BF16 rsfde_apply_precond alone waits for it).  In FP64
+ * a device-side wait that gives up in rsfde_apply_M, rsfde_apply_precond or
+ * rsfde_dst2 therefore shows in the values it left incomplete, which are NaN; a later solve
+ * reports its own give-ups only. */
 /* Eq. 2.14-2.17: w = M z in the context's operator precision (matvec_prec).
  * z, w device N doubles (distinct). */
 int rsfde_apply_M(rsfde_ctx* ctx, const double* z, double* w);
@@ -260,9 +265,7 @@ int rsfde_apply_M(rsfde_ctx* ctx, const double* z, double* w);
  * resid_prec, RSFDE_FP64 or RSFDE_EXACT (RSFDE_DF32: RSFDE_EINVAL).  x, b, r
  * device N doubles (r distinct from x and b). */
 int rsfde_residual(rsfde_ctx* ctx, const double* x, const double* b, double* r);
-/* Eq. 4.6: z = P-hat^-1 v in the context's preconditioner precision (result in FP64).
- * (FP64, and rsfde_dst2: if a device-side wait gives up, the values it left
- * incomplete are NaN, and the next solve or step returns RSFDE_ETIMEOUT.) */
+/* Eq. 4.6: z = P-hat^-1 v in the context's preconditioner precision (result in FP64). */
 int rsfde_apply_precond(rsfde_ctx* ctx, const double* v, double* z);
 /* Section 4.1: out = (S_{n2} (x) S_{n1}) v, the orthonormal 2D sine transform, FP64. */
 int rsfde_dst2(rsfde_ctx* ctx, const double* v, double* out);
@@ -357,13 +360,14 @@ int rsfde_batch_autotune(rsfde_batch* b, int32_t reps);
 /* Failure detection.  Every wait of the tensor-core preconditioners'
  * pipeline (a TMA copy landing in a ring slot, a slot freed by the MMAs) is
  * bounded; a wait that runs out makes that launch give up and the call
- * return RSFDE_ETIMEOUT, after every copy and MMA the launch had issued has
+ * (the operator-level ones in FP64 aside, see there) return RSFDE_ETIMEOUT, after every copy and MMA the launch had issued has
  * completed, so the context stays usable.  cycles: the bound of each such
  * wait in SM clock cycles; 0 restores the default (4e9, about 2 s at
  * 2.07 GHz).  A small bound makes the waits give up on purpose, which is how
  * the timeout path is tested.  The waits that let issued work complete
  * before a block frees its memory keep the default bound. */
 int rsfde_set_wait_cycles(rsfde_ctx* ctx, int64_t cycles);
+int rsfde_batch_set_wait_cycles(rsfde_batch* b, int64_t cycles); /* of every instance */
 
 /* Number of this library's kernel launches since the context was made (host counter). */
 int64_t rsfde_kernel_launches(const rsfde_ctx* ctx);

@@ -120,6 +120,8 @@ def load_library(path=LIB_PATH):
     lib.rsfde_batch_kernel_launches.argtypes = [vp]
     lib.rsfde_batch_kernel_launches.restype = ctypes.c_int64
     lib.rsfde_batch_destroy.argtypes = [vp]
+    lib.rsfde_batch_set_wait_cycles.argtypes = [vp, ctypes.c_int64]
+    lib.rsfde_batch_set_wait_cycles.restype = ctypes.c_int
     lib.rsfde_autotune.argtypes = [vp, i32, vp]
     lib.rsfde_autotune.restype = ctypes.c_int
     lib.rsfde_batch_autotune.argtypes = [vp, i32]
@@ -435,6 +437,10 @@ class Batch:
         rc = self._lib.rsfde_batch_run(self._h, int(steps), st)
         _check(rc, "batch_run")
         return [x.as_dict() for x in st]
+
+    def set_wait_cycles(self, cycles=0):
+        """Solver.set_wait_cycles of every instance."""
+        _check(self._lib.rsfde_batch_set_wait_cycles(self._h, int(cycles)), "batch_set_wait_cycles")
 
     def autotune(self, reps=3):
         _check(self._lib.rsfde_batch_autotune(self._h, int(reps)), "batch_autotune")

@@ -430,7 +430,7 @@ bool left_variant(const rsfde_ctx* c) { return c->opts.variant == RSFDE_GMRES_LE
 // 512 55 / 93, 2048 x 2048 0.51 ms / 1.53.
 int ensure_digit_operator(rsfde_ctx* c) {
   if (c->dop || c->opts.matvec_prec != RSFDE_FP64 || left_variant(c) || !digit_sizes_ok(c->n1, c->n2)) return RSFDE_OK;
-  if (digit_operator_create(&c->dop, c->n1, c->n2, c->stream) != RSFDE_OK) return RSFDE_OK;
+  if (digit_operator_create(&c->dop, c->n1, c->n2, &c->st->gave_up, c->stream) != RSFDE_OK) return RSFDE_OK;
   if (!digit_operator_params(c->dop, c->hx_axis.t, c->hy_axis.t, c->stream)) {
     take_launch_error();
     digit_operator_destroy(c->dop);
@@ -449,7 +449,7 @@ int ensure_digits(rsfde_ctx* c) {
   if (c->digit || c->opts.precond_prec != RSFDE_FP64 || !c->opts.use_precond || left_variant(c) ||
       !digit_sizes_ok(c->n1, c->n2))
     return RSFDE_OK;
-  if (digit_plan_create(&c->digit, c->n1, c->n2, c->stream) != RSFDE_OK) return RSFDE_OK;
+  if (digit_plan_create(&c->digit, c->n1, c->n2, &c->st->gave_up, c->stream) != RSFDE_OK) return RSFDE_OK;
   digit_plan_params(c->digit, c->x64.tab.lam, c->y64.tab.lam, c->pen, c->stream);
   digit_plan_set_wait(c->digit, c->wait_cycles);
   return RSFDE_OK;
@@ -676,9 +676,9 @@ double rhs_bytes(const rsfde_ctx* c, bool has_uu, bool has_src) {
   return (8.0 + (has_uu ? 8.0 : 0.0) + (has_src ? 8.0 : 0.0) + 16.0) * N + N / 8.0;
 }
 
-void enqueue_init(rsfde_ctx* c) {
+void enqueue_init(rsfde_ctx* c, bool own = true) {
   ProfScope ps(c, RSFDE_K_OTHER);
-  launch_init_state(c->st, c->opts.restart, c->opts.max_iter, c->opts.tol, c->stream);
+  launch_init_state(c->st, c->opts.restart, c->opts.max_iter, c->opts.tol, own, c->stream);
 }
 
 void enqueue_rhs(rsfde_ctx* c, const double* u, const double* uu, const double* src, double* b, double* x0) {
@@ -927,9 +927,7 @@ int run_solver(rsfde_ctx* c, rsfde_stats* stats) {
   const SolverState& h = *c->st_host;
   if (c->opts.use_graph && !c->prof_on) c->launches += (int64_t)h.body_runs * c->launches_per_body;
   if (c->bf16 && bf16_precond_on(c) && (rc = bf16_plan_error(c->bf16, c->stream))) return rc;
-  const int e1 = digit_precond_on(c) ? digit_plan_error(c->digit, c->stream) : RSFDE_OK;
-  const int e2 = digit_operator_on(c) ? digit_operator_error(c->dop, c->stream) : RSFDE_OK;
-  if (e1 || e2) return e1 ? e1 : e2;
+  if (h.gave_up) return RSFDE_ETIMEOUT;
   if (stats) {
     stats->iters = h.iters;
     stats->restarts = h.cycles > 0 ? h.cycles - 1 : 0;
@@ -1604,7 +1602,7 @@ int build_batch_graph(rsfde_batch* b, int later) {
     const int64_t l0 = c->launches;
     e = add_captured(c, g, nullptr, 0,
                      [&](rsfde_ctx* cc) {
-                       enqueue_init(cc);
+                       enqueue_init(cc, false);
                        enqueue_rhs(cc, u_prev, later ? u_pp : nullptr, src, cc->b, cc->x);
                        if (left_variant(cc)) enqueue_bnorm(cc);
                        enqueue_residual(cc, &cc->st->run_cycle);
@@ -2119,11 +2117,19 @@ int rsfde_batch_run(rsfde_batch* b, int32_t steps, rsfde_stats* stats) {
     e = cudaMemcpy(c->st_host, c->st, head, cudaMemcpyDeviceToHost);
     if (e != cudaSuccess) return cuda_fail(e);
     const SolverState& h = *c->st_host;
+    int gave_up = h.gave_up ? RSFDE_ETIMEOUT : RSFDE_OK;  // in one of the run's steps
+    if (gave_up && (e = cudaMemset(&c->st->gave_up, 0, sizeof(int))) != cudaSuccess) return cuda_fail(e);
+    if (!b->multi && bf16_precond_on(c)) {  // an instance's own split-BF16 or BF16 GEMMs
+      const int rc = bf16_plan_error(c->bf16, b->stream);
+      if (rc != RSFDE_OK && rc != RSFDE_ETIMEOUT) return rc;
+      if (rc) gave_up = rc;
+    }
+    if (gave_up) worst = gave_up;
     if (stats) {
       stats[i].iters = h.iters;
       stats[i].restarts = h.cycles > 0 ? h.cycles - 1 : 0;
       stats[i].converged = h.converged;
-      stats[i].status = h.status;
+      stats[i].status = gave_up ? gave_up : h.status;
       stats[i].rel_res = 0.0;
       stats[i].bnorm = 0.0;
       for (int k = 0; k < 6; ++k) stats[i].t_ms[k] = 0.0;
@@ -2142,6 +2148,19 @@ int rsfde_batch_run(rsfde_batch* b, int32_t steps, rsfde_stats* stats) {
     }
   }
   return worst;
+}
+
+int rsfde_batch_set_wait_cycles(rsfde_batch* b, int64_t cycles) {
+  if (!b || cycles < 0) return RSFDE_EINVAL;
+  for (rsfde_ctx* c : b->ctx) rsfde_set_wait_cycles(c, cycles);
+  if (b->bf16) return bf16_group_set_wait(b->gdesc, b->count, cycles);
+  if (!b->multi)
+    for (auto& x : b->exec)
+      if (x) {  // captured launches carry the old bound
+        cudaGraphExecDestroy(x);
+        x = nullptr;
+      }
+  return RSFDE_OK;
 }
 
 int rsfde_batch_get(rsfde_batch* b, int32_t i, double* u_out) {

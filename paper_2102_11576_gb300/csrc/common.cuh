@@ -52,6 +52,7 @@ struct SolverState {
   int iters, cycles, max_iter, m;
   int zero_solution;  // b == 0: x must be zeroed
   int body_runs;      // FGMRES cycles replayed by the device-side graph loop (this solve)
+  int gave_up;        // 1 once a wait of an FP64 digit product gave up (cleared by the host's calls)
   long long total_body_runs;  // the same over the context's lifetime (never reset)
   long long sum_j;            // sum of the Arnoldi column index j over the solve's iterations
   unsigned int counter;  // arrivals for the last-block reductions

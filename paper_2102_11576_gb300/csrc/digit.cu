@@ -380,7 +380,8 @@ struct DigitPlan {
   int kx = 0, ky = 0;            // scale of a product with S_x, S_y (DigitEpiParams::kexp)
   double* inv = nullptr;         // the two tables of reciprocals (N each)
   int* exps = nullptr;           // row exponents: n2 (A0), n1 (T), 2 n2 (W), 2 n1 (Y)
-  int* err = nullptr;            // give-up flags (digit_gemm_kernel), and a word for the setup
+  int* err = nullptr;            // an application's give-up flag (digit_gemm_kernel), and a word for the setup
+  int* gave_up = nullptr;        // the context's
   void* mem = nullptr;
   long long wait_cycles = kWaitCycles;
 };
@@ -419,11 +420,12 @@ static bool build_sine(DigitMat* S, int n, long long* tab_dev, int* rowsum_dev, 
 
 bool digit_sizes_ok(int n1, int n2) { return n1 <= kDgMaxN && n2 <= kDgMaxN; }
 
-int digit_plan_create(DigitPlan** out, int n1, int n2, cudaStream_t s) {
+int digit_plan_create(DigitPlan** out, int n1, int n2, int* gave_up, cudaStream_t s) {
   *out = nullptr;
   if (!digit_sizes_ok(n1, n2)) return RSFDE_EINVAL;
   DigitPlan* p = new (std::nothrow) DigitPlan();
   if (!p) return RSFDE_ENOMEM;
+  p->gave_up = gave_up;
   p->n1 = n1;
   p->n2 = n2;
   const int h1 = pad16((n1 + 1) / 2), h2 = pad16((n2 + 1) / 2);
@@ -458,9 +460,9 @@ int digit_plan_create(DigitPlan** out, int n1, int n2, cudaStream_t s) {
   long long* tab = reinterpret_cast<long long*>(b + sx + sy + sw + si + se + 256);
   bool good = cudaMemsetAsync(p->err, 0, 256, s) == cudaSuccess &&
               cudaMemsetAsync(p->exps, 0, nexp * sizeof(int), s) == cudaSuccess;
-  good = good && build_sine(&p->Sx, n1, tab, p->err + 2, &p->kx, s);
+  good = good && build_sine(&p->Sx, n1, tab, p->err + 1, &p->kx, s);
   p->ky = p->kx;
-  if (n1 != n2) good = good && build_sine(&p->Sy, n2, tab, p->err + 2, &p->ky, s);
+  if (n1 != n2) good = good && build_sine(&p->Sy, n2, tab, p->err + 1, &p->ky, s);
   for (DigitMat* m : {&p->A0, &p->T, &p->W, &p->Y}) good = good && digit_map(m, &m->map[0], kDgBM, 1);
   for (DigitMat* m : {&p->Sx, &p->Sy})
     for (int k = 0; k < 3; ++k) good = good && digit_map(m, &m->map[k], 64 >> k, kDgDigits);
@@ -483,15 +485,6 @@ void digit_plan_params(DigitPlan* p, const double* lamx, const double* lamy, dou
   const size_t N = (size_t)p->n1 * p->n2;
   digit_reciprocals_kernel<<<vec_grid(N), kBlock, 0, s>>>(lamx, lamy, pen, p->n1, p->n2, p->inv, p->inv + N);
 }
-
-static int digit_error(int* err, cudaStream_t s) {
-  int h = 0;
-  if (cudaMemcpyAsync(&h, err + 1, sizeof(int), cudaMemcpyDeviceToHost, s) != cudaSuccess) return RSFDE_ECUDA;
-  if (cudaStreamSynchronize(s) != cudaSuccess) return RSFDE_ECUDA;
-  if (h && cudaMemsetAsync(err, 0, 2 * sizeof(int), s) != cudaSuccess) return RSFDE_ECUDA;
-  return h ? RSFDE_ETIMEOUT : RSFDE_OK;
-}
-int digit_plan_error(DigitPlan* p, cudaStream_t s) { return digit_error(p->err, s); }
 
 void digit_plan_set_wait(DigitPlan* p, long long cycles) {
   if (p) p->wait_cycles = cycles > 0 ? cycles : kWaitCycles;
@@ -564,6 +557,7 @@ static void launch_digit(const Plan* p, const DigitMat& A, const DigitMat& S, in
   ep.hk = A.hk;
   ep.kexp = kexp;
   ep.wait_cycles = p->wait_cycles;
+  ep.gave_up = p->gave_up;
   const int bn = dg_bn(ep.N, ep.M, ep.hk);
   ep.early = next == 0 || (ep.N + bn - 1) / bn * ((ep.M + kDgBM - 1) / kDgBM) + next <= kNumSMs;
   if (bn == 64) launch_digit_bn<EPI, 64>(A, S, ep, p->err, gate, s);
@@ -647,6 +641,7 @@ struct DigitOperator {
   DigitMat Tx, Ty, R, C;  // [U | V] of each axis; the rows and the columns of z
   int* exps = nullptr;     // n2 (rows), n1 (columns)
   int* err = nullptr;
+  int* gave_up = nullptr;
   // the parameters, on the device (captured launches read them where they are):
   double* near = nullptr;  // 1 - t0x - t0y, t1x, t1y
   int* kexp = nullptr;     // the scales of the two products
@@ -668,10 +663,10 @@ static bool build_toeplitz(DigitOperator* p, DigitMat* T, const std::vector<doub
     for (int k = 2; k < n; ++k) q[k] = std::llround(std::ldexp(t[k], sh));
     int rowsum = 0;
     if (cudaMemcpyAsync(p->tq, q.data(), n * sizeof(long long), cudaMemcpyHostToDevice, s) != cudaSuccess ||
-        cudaMemsetAsync(p->err + 2, 0, sizeof(int), s) != cudaSuccess)
+        cudaMemsetAsync(p->err + 1, 0, sizeof(int), s) != cudaSuccess)
       return false;
-    digit_toeplitz_kernel<<<T->rows, 256, 0, s>>>(p->tq, n, T->d, T->plane(), T->hk, p->err + 2);
-    if (cudaMemcpyAsync(&rowsum, p->err + 2, sizeof(int), cudaMemcpyDeviceToHost, s) != cudaSuccess ||
+    digit_toeplitz_kernel<<<T->rows, 256, 0, s>>>(p->tq, n, T->d, T->plane(), T->hk, p->err + 1);
+    if (cudaMemcpyAsync(&rowsum, p->err + 1, sizeof(int), cudaMemcpyDeviceToHost, s) != cudaSuccess ||
         cudaStreamSynchronize(s) != cudaSuccess)
       return false;
     // z = z_q 2^(E_z - 1077), 2U = U_q 2^-sh, sum z U = W 2^(9 + 49 - 1) 2^(E_z - 1077 - sh)
@@ -691,11 +686,12 @@ bool digit_operator_params(DigitOperator* p, const std::vector<double>& tx, cons
          cudaStreamSynchronize(s) == cudaSuccess;
 }
 
-int digit_operator_create(DigitOperator** out, int n1, int n2, cudaStream_t s) {
+int digit_operator_create(DigitOperator** out, int n1, int n2, int* gave_up, cudaStream_t s) {
   *out = nullptr;
   if (!digit_sizes_ok(n1, n2)) return RSFDE_EINVAL;
   DigitOperator* p = new (std::nothrow) DigitOperator();
   if (!p) return RSFDE_ENOMEM;
+  p->gave_up = gave_up;
   p->n1 = n1;
   p->n2 = n2;
   const int h1 = pad16((n1 + 1) / 2), h2 = pad16((n2 + 1) / 2);
@@ -738,7 +734,6 @@ void digit_operator_destroy(DigitOperator* p) {
   if (p->mem) cudaFree(p->mem);
   delete p;
 }
-int digit_operator_error(DigitOperator* p, cudaStream_t s) { return digit_error(p->err, s); }
 void digit_operator_set_wait(DigitOperator* p, long long cycles) {
   if (p) p->wait_cycles = cycles > 0 ? cycles : kWaitCycles;
 }

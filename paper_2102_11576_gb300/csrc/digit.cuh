@@ -86,6 +86,7 @@ struct DigitEpiParams {
   double pen;          // dt/eta
   int early;           // trigger the next kernel of the chain at once (launch_digit)
   long long wait_cycles;
+  int* gave_up;        // set when a wait gave up
 };
 
 // Digits of x_q (|x_q| <= 2^55): x_q + sum_i 64 128^i has the base-128 digits
@@ -356,9 +357,8 @@ __global__ void __launch_bounds__(kDgThreads, 1)
     ok = mbar_wait(&done[1], 0, err) && ok;
     tc_fence_after();
   }
-  // err[0]: a wait of this application's launches gave up; err[1]: one did since the host last looked
-  const bool bad = !ok || *(volatile int*)err != 0;
-  if (bad && lane == 0) atomicExch(err + 1, 1);
+  const bool bad = !ok || *(volatile int*)err != 0;  // *err: a wait of this application's launches gave up
+  if (bad && lane == 0) atomicExch(ep.gave_up, 1);
   const int kexp = ep.kexp + kdev, kx = E + kexp;
   const bool nan = bad || E == kDgNan;  // an incomplete tile, or a row that held an infinity or NaN
   const bool ch = m >= ep.row_b;

@@ -520,6 +520,13 @@ int bf16_group_create(const std::vector<Bf16GroupInst>& in, void** descs, std::v
   }
   return RSFDE_OK;
 }
+int bf16_group_set_wait(void* descs, int count, long long cycles) {
+  const std::vector<long long> w(4 * (size_t)count, cycles > 0 ? cycles : kWaitCycles);
+  char* at = static_cast<char*>(descs) + offsetof(GemmGroupDesc, ep) + offsetof(GemmEpiParams, wait_cycles);
+  const cudaError_t e = cudaMemcpy2D(at, sizeof(GemmGroupDesc), w.data(), sizeof(w[0]), sizeof(w[0]), w.size(),
+                                     cudaMemcpyHostToDevice);
+  return e == cudaSuccess ? RSFDE_OK : RSFDE_ECUDA;
+}
 void bf16_group_destroy(void* descs) {
   if (descs) cudaFree(descs);
 }

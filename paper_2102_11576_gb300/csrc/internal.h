@@ -209,11 +209,11 @@ bool bf16_plan_a0(const Bf16Plan* p, int vec, Bf16Out* out);
 // ---- FP64 sine transforms as digit products on the tensor cores (digit.cu) ---
 struct DigitPlan;
 bool digit_sizes_ok(int n1, int n2);  // the sides the digit products take (both <= 2048)
-int digit_plan_create(DigitPlan** out, int n1, int n2, cudaStream_t s);
+// gave_up: device word that a wait that gives up sets
+int digit_plan_create(DigitPlan** out, int n1, int n2, int* gave_up, cudaStream_t s);
 void digit_plan_destroy(DigitPlan* p);
 // the tabulated reciprocals of the tau divides (enqueued on s)
 void digit_plan_params(DigitPlan* p, const double* lamx, const double* lamy, double pen, cudaStream_t s);
-int digit_plan_error(DigitPlan* p, cudaStream_t s);  // reads and clears the give-up flag
 void digit_plan_set_wait(DigitPlan* p, long long cycles);  // <= 0: the default bound
 // z = P-hat^-1 (scale v) in eight launches; t, wa, wb: N doubles of scratch each
 template <typename Tin>
@@ -226,11 +226,10 @@ void digit_dst2(DigitPlan* p, const double* v, double* out, double* t, cudaStrea
 // scratch.  Tables from the Toeplitz columns (digit_operator_params:
 // false if no scale keeps the sums exact).
 struct DigitOperator;
-int digit_operator_create(DigitOperator** out, int n1, int n2, cudaStream_t s);
+int digit_operator_create(DigitOperator** out, int n1, int n2, int* gave_up, cudaStream_t s);
 void digit_operator_destroy(DigitOperator* p);
 bool digit_operator_params(DigitOperator* p, const std::vector<double>& tx, const std::vector<double>& ty,
                            cudaStream_t s);
-int digit_operator_error(DigitOperator* p, cudaStream_t s);
 void digit_operator_set_wait(DigitOperator* p, long long cycles);
 template <typename Tin>
 void digit_apply_M(DigitOperator* p, const Tin* z, double* w, const uint8_t* phi, double pen, double* pre,
@@ -411,6 +410,7 @@ struct Bf16GroupInst {
 // counts per instance of each GEMM (the grids of the grouped launches).
 int bf16_group_create(const std::vector<Bf16GroupInst>& in, void** descs, std::vector<int>* tiles);
 void bf16_group_destroy(void* descs);
+int bf16_group_set_wait(void* descs, int count, long long cycles);  // <= 0: the default bound
 void launch_bf16_group(int k, const void* descs, int count, const int* active, int max_tiles, int j, int* err,
                        cudaStream_t s);
 void launch_split_multi(const BatchInst* bi, const MultiGrid& g, int j, cudaStream_t s);
@@ -439,7 +439,7 @@ int xupdate_blocks(size_t N, int zbytes);
 
 // ---- launchers (krylov.cu) -------------------------------------------------
 int vec_grid(size_t N);
-void launch_init_state(SolverState* st, int m, int max_iter, double tol, cudaStream_t s);
+void launch_init_state(SolverState* st, int m, int max_iter, double tol, int own, cudaStream_t s);
 void launch_mask_to_phi(const uint8_t* in_omega, uint8_t* phi, size_t N, cudaStream_t s);
 void launch_rhs(const double* u, const double* uu, const double* src, const uint8_t* phi, double dt, double* b,
                 double* x0, size_t N, double* partials, SolverState* st, cudaStream_t s);

@@ -45,8 +45,10 @@ __device__ __forceinline__ void init_state_body(SolverState* st, int m, int max_
   st->beta = 0.0;
   st->rel_res = 0.0;
 }
-__global__ void init_state_kernel(SolverState* st, int m, int max_iter, double tol) {
+// own: a solve of its own, which reports its own give-ups (a batch's step leaves them for the run's end)
+__global__ void init_state_kernel(SolverState* st, int m, int max_iter, double tol, int own) {
   init_state_body(st, m, max_iter, tol);
+  if (own) st->gave_up = 0;
 }
 
 __global__ void mask_to_phi_kernel(const uint8_t* __restrict__ in_omega, uint8_t* __restrict__ phi, size_t N) {
@@ -812,8 +814,8 @@ __global__ void __launch_bounds__(kBlock) xupdate_v_kernel(double* __restrict__ 
 }
 
 // ---- launchers --------------------------------------------------------------
-void launch_init_state(SolverState* st, int m, int max_iter, double tol, cudaStream_t s) {
-  init_state_kernel<<<1, 1, 0, s>>>(st, m, max_iter, tol);
+void launch_init_state(SolverState* st, int m, int max_iter, double tol, int own, cudaStream_t s) {
+  init_state_kernel<<<1, 1, 0, s>>>(st, m, max_iter, tol, own);
 }
 void launch_mask_to_phi(const uint8_t* in_omega, uint8_t* phi, size_t N, cudaStream_t s) {
   mask_to_phi_kernel<<<vec_grid(N), kBlock, 0, s>>>(in_omega, phi, N);
