@@ -1065,7 +1065,7 @@ int autotune_ctx(rsfde_ctx* c, int reps, int32_t* chosen_out) {
   } else if (c->opts.matvec_prec == RSFDE_FP32) {
     if (b64) tune_operator<float, double>(c, reps, c->x32.tab, c->y32.tab, chosen);
     else tune_operator<float, float>(c, reps, c->x32.tab, c->y32.tab, chosen);
-  } else if (!digit_operator_on(c)) {
+  } else {  // (beside digit products: the FFTs of rsfde_residual and the adjoint)
     tune_operator<double, double>(c, reps, c->x64.tab, c->y64.tab, chosen);
   }
   // the double-FP32 true residual runs the same transform families in 8-byte
@@ -1075,7 +1075,7 @@ int autotune_ctx(rsfde_ctx* c, int reps, int32_t* chosen_out) {
     tune_residual<df>(c, reps, c->xdf.tab, c->ydf.tab, unused);
   }
   if (c->opts.precond_prec == RSFDE_FP32) tune_precond<float>(c, reps, c->x32.tab, c->y32.tab, chosen);
-  else if (c->opts.precond_prec == RSFDE_FP64 && !digit_precond_on(c))
+  else if (c->opts.precond_prec == RSFDE_FP64)
     tune_precond<double>(c, reps, c->x64.tab, c->y64.tab, chosen);
   int bn[4] = {0, 0, 0, 0};
   int rc = RSFDE_OK;

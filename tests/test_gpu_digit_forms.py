@@ -56,3 +56,11 @@ def test_operators_in_place(n1, n2):
         ref, x = op(v), v.clone()
         assert torch.equal(op(x, out=x), ref)
     s.close()
+
+
+def test_autotune_still_takes_the_fp64_transforms():
+    w = workloads.random_problem(72, 100, 70)
+    s = solver(w)
+    chosen = s.autotune(reps=1)  # rsfde_residual and the adjoint run them beside the digit products
+    assert {"toeplitz_rows", "toeplitz_cols", "dst_rows", "precond_cols", "precond_rows"} <= set(chosen)
+    s.close()
