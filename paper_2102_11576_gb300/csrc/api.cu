@@ -244,6 +244,7 @@ struct rsfde_ctx {
   int64_t launches = 0;
   Bf16Plan* bf16 = nullptr;  // tensor-core preconditioner, made when first needed
   DigitPlan* digit = nullptr;  // FP64 preconditioner as digit products (nullptr: FP64 FFTs)
+  bool digit_refused = false;    // the sides have no digit products: not tried again
   DigitOperator* dop = nullptr;  // FP64 operator likewise
   long long wait_cycles = 0;  // their pipeline wait bound (0: the default)
   // one FGMRES cycle captured as the body of a device-side WHILE loop
@@ -446,10 +447,11 @@ bool digit_operator_on(const rsfde_ctx* c) {
 int ensure_digits(rsfde_ctx* c) {
   const int rc = ensure_digit_operator(c);
   if (rc != RSFDE_OK) return rc;
-  if (c->digit || c->opts.precond_prec != RSFDE_FP64 || !c->opts.use_precond || left_variant(c) ||
-      !digit_sizes_ok(c->n1, c->n2))
+  if (c->digit || c->digit_refused || c->opts.precond_prec != RSFDE_FP64 || !c->opts.use_precond || left_variant(c))
     return RSFDE_OK;
-  if (digit_plan_create(&c->digit, c->n1, c->n2, &c->st->gave_up, c->stream) != RSFDE_OK) return RSFDE_OK;
+  const int made = digit_plan_create(&c->digit, c->n1, c->n2, &c->st->gave_up, c->stream);
+  c->digit_refused = made == RSFDE_EINVAL;
+  if (made != RSFDE_OK) return RSFDE_OK;
   digit_plan_params(c->digit, c->x64.tab.lam, c->y64.tab.lam, c->pen, c->stream);
   digit_plan_set_wait(c->digit, c->wait_cycles);
   return RSFDE_OK;

@@ -386,9 +386,13 @@ struct DigitPlan {
   long long wait_cycles = kWaitCycles;
 };
 
-// S_n as digits; *kexp the scale of a product with it.  False: no scale keeps
-// the accumulators exact, or a CUDA call failed.
-static bool build_sine(DigitMat* S, int n, long long* tab_dev, int* rowsum_dev, int* kexp, cudaStream_t s) {
+// S_n as digits; *kexp the scale of a product with it.  RSFDE_EINVAL: none of the
+// scales keeps the accumulators exact.  So it is for 21 of the sides up to 2048: 1869, 1895,
+// 1907, 1915, 1919, 1931, 1947, 1959, 1963, 1969, 1975, 1979, 1983, 1987, 1991, 1999, 2015, 2023, 2031,
+// 2039 and 2047.  There n + 1 has divisors d such that some rows' sines take few values; one
+// magnitude then stands in most of half a row, and if its digits sum to more than about 256 they
+// are not averaged over the row as other rows' are.
+static int build_sine(DigitMat* S, int n, long long* tab_dev, int* rowsum_dev, int* kexp, cudaStream_t s) {
   const long per = 2L * (n + 1);
   std::vector<long long> tab(per);
   const long double sc = sqrtl(2.0L / (n + 1));
@@ -406,16 +410,16 @@ static bool build_sine(DigitMat* S, int n, long long* tab_dev, int* rowsum_dev, 
     int rowsum = 0;
     if (cudaMemcpyAsync(tab_dev, tab.data(), per * sizeof(long long), cudaMemcpyHostToDevice, s) != cudaSuccess ||
         cudaMemsetAsync(rowsum_dev, 0, sizeof(int), s) != cudaSuccess)
-      return false;
+      return RSFDE_ECUDA;
     digit_sine_kernel<<<S->rows, 256, 0, s>>>(tab_dev, n, S->d, S->plane(), S->hk, rowsum_dev);
     if (cudaMemcpyAsync(&rowsum, rowsum_dev, sizeof(int), cudaMemcpyDeviceToHost, s) != cudaSuccess ||
         cudaStreamSynchronize(s) != cudaSuccess)
-      return false;
+      return RSFDE_ECUDA;
     // x = x_q 2^(E_x - 1077), S = S_q 2^-sh, sum x S = W 2^(9 + 49) 2^(E_x - 1077 - sh)
     *kexp = 58 - 1077 - sh;
-    if (64LL * rowsum <= (1LL << 24)) return true;
+    if (64LL * rowsum <= (1LL << 24)) return RSFDE_OK;
   }
-  return false;
+  return RSFDE_EINVAL;
 }
 
 bool digit_sizes_ok(int n1, int n2) { return n1 <= kDgMaxN && n2 <= kDgMaxN; }
@@ -460,16 +464,17 @@ int digit_plan_create(DigitPlan** out, int n1, int n2, int* gave_up, cudaStream_
   long long* tab = reinterpret_cast<long long*>(b + sx + sy + sw + si + se + 256);
   bool good = cudaMemsetAsync(p->err, 0, 256, s) == cudaSuccess &&
               cudaMemsetAsync(p->exps, 0, nexp * sizeof(int), s) == cudaSuccess;
-  good = good && build_sine(&p->Sx, n1, tab, p->err + 1, &p->kx, s);
+  int rc = good ? build_sine(&p->Sx, n1, tab, p->err + 1, &p->kx, s) : RSFDE_ECUDA;
   p->ky = p->kx;
-  if (n1 != n2) good = good && build_sine(&p->Sy, n2, tab, p->err + 1, &p->ky, s);
+  if (n1 != n2 && rc == RSFDE_OK) rc = build_sine(&p->Sy, n2, tab, p->err + 1, &p->ky, s);
+  good = rc == RSFDE_OK;
   for (DigitMat* m : {&p->A0, &p->T, &p->W, &p->Y}) good = good && digit_map(m, &m->map[0], kDgBM, 1);
   for (DigitMat* m : {&p->Sx, &p->Sy})
     for (int k = 0; k < 3; ++k) good = good && digit_map(m, &m->map[k], 64 >> k, kDgDigits);
   if (!good) {
     take_launch_error();
     digit_plan_destroy(p);
-    return RSFDE_ECUDA;
+    return rc != RSFDE_OK ? rc : RSFDE_ECUDA;
   }
   *out = p;
   return RSFDE_OK;

@@ -209,7 +209,8 @@ bool bf16_plan_a0(const Bf16Plan* p, int vec, Bf16Out* out);
 // ---- FP64 sine transforms as digit products on the tensor cores (digit.cu) ---
 struct DigitPlan;
 bool digit_sizes_ok(int n1, int n2);  // the sides the digit products take (both <= 2048)
-// gave_up: device word that a wait that gives up sets
+// gave_up: device word that a wait that gives up sets.  RSFDE_EINVAL: the sides have no digit
+// products (beyond 2048, or no scale keeps their sums exact); other errors may pass.
 int digit_plan_create(DigitPlan** out, int n1, int n2, int* gave_up, cudaStream_t s);
 void digit_plan_destroy(DigitPlan* p);
 // the tabulated reciprocals of the tau divides (enqueued on s)

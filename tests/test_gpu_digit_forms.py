@@ -1,4 +1,6 @@
 """The FP64 forms' digit products on what test_gpu_digit.py does not reach."""
+import time
+
 import numpy as np
 import pytest
 
@@ -64,3 +66,19 @@ def test_autotune_still_takes_the_fp64_transforms():
     chosen = s.autotune(reps=1)  # rsfde_residual and the adjoint run them beside the digit products
     assert {"toeplitz_rows", "toeplitz_cols", "dst_rows", "precond_cols", "precond_rows"} <= set(chosen)
     s.close()
+
+
+def test_sides_without_digit_products_are_tried_once():
+    """A try makes three tables of 4,096 long-double sines and waits for three kernels."""
+    took = {}
+    for n1 in (2047, 2048):  # no scale of S_2047's digits keeps the sums exact
+        w = workloads.random_problem(73, n1, 5)
+        s = solver(w)
+        calls = []
+        for _ in range(20):
+            t = time.perf_counter()
+            s.set_options(tol=1e-10)
+            calls.append(time.perf_counter() - t)
+        took[n1] = min(calls)
+        s.close()
+    assert took[2047] <= 5 * took[2048]
