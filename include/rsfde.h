@@ -262,7 +262,8 @@ void rsfde_batch_destroy(rsfde_batch* b);
  * z, w device N doubles (distinct). */
 int rsfde_apply_M(rsfde_ctx* ctx, const double* z, double* w);
 /* The true residual r = b - M x (Eq. 2.17's system) with M x in the context's
- * resid_prec, RSFDE_FP64 or RSFDE_EXACT (RSFDE_DF32: RSFDE_EINVAL).  x, b, r
+ * resid_prec, RSFDE_FP64 or RSFDE_EXACT (RSFDE_DF32: RSFDE_EINVAL).  RSFDE_FP64: by FFTs, also where a
+ * solve's own test takes M x from the FP64 digit products, so the two agree to rounding.  x, b, r
  * device N doubles (r distinct from x and b). */
 int rsfde_residual(rsfde_ctx* ctx, const double* x, const double* b, double* r);
 /* Eq. 4.6: z = P-hat^-1 v in the context's preconditioner precision (result in FP64). */
@@ -311,7 +312,8 @@ int rsfde_dst2_noalloc(int32_t n1, int32_t n2, const double* v, double* out, voi
 /* ---- measurement ------------------------------------------------------------ */
 /* Kernel classes timed by the profiler. */
 #define RSFDE_K_TOEPLITZ_ROWS 0 /* (I (x) A_x) z, Eq. 2.15 */
-#define RSFDE_K_TOEPLITZ_COLS 1 /* (A_y (x) I) z fused with the rest of M (or the residual) */
+#define RSFDE_K_TOEPLITZ_COLS 1 /* (A_y (x) I) z fused with the rest of M (or the residual); the whole of M z
+                                   where FP64 runs as digit products (then no launch is TOEPLITZ_ROWS) */
 #define RSFDE_K_DST_ROWS 2      /* first row sine transform of Eq. 4.6 */
 #define RSFDE_K_PRECOND_COLS 3  /* column sine transforms and tau divides of Eq. 4.6 */
 #define RSFDE_K_PRECOND_ROWS 4  /* last row sine transforms and the masked combine of Eq. 4.6 */
@@ -322,10 +324,14 @@ int rsfde_dst2_noalloc(int32_t n1, int32_t n2, const double* v, double* out, voi
 #define RSFDE_K_DST_GEMM 9      /* preconditioner (and rsfde_dst2) as tensor-core GEMMs: split-BF16 or
                                    BF16 (the four GEMMs and, when the previous Gram-Schmidt update did
                                    not write the first operand, the split), or FP64 by digit products
-                                   (four splits and four products; sides up to 2048, not in paper mode:
-                                   there, and beyond, FP64 runs as FFTs) */
-#define RSFDE_K_RESID_ROWS 10   /* row pass of M x in the true residual (Eq. 2.15) */
-#define RSFDE_K_RESID_COLS 11   /* column pass of the true residual b - M x and its norm */
+                                   (four splits and four products).  FP64 FFTs, whose launches are
+                                   DST_ROWS and the two after it, run in paper mode, beyond 2048 a
+                                   side, where the digits' tables find no memory (0.23 GB at 2048 x 2048,
+                                   the operator's 0.20 GB), and, the operator aside, with a side of 1869,
+                                   1895, 1907, 1915, 1919, 1931, 1947, 1959, 1963, 1969, 1975, 1979, 1983,
+                                   1987, 1991, 1999, 2015, 2023, 2031, 2039 or 2047, whose sines no digits keep exact */
+#define RSFDE_K_RESID_ROWS 10   /* row pass of M x in the true residual (Eq. 2.15), or M x by digit products */
+#define RSFDE_K_RESID_COLS 11   /* column pass of the true residual b - M x (or the difference) and its norm */
 #define RSFDE_K_SOLVE_Y 12      /* back substitution of the Givens-rotated least squares */
 #define RSFDE_K_COUNT 13
 

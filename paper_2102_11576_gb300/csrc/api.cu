@@ -419,10 +419,10 @@ int ensure_bf16(rsfde_ctx* c) {
 }
 
 // The FP64 preconditioner runs as digit products on the tensor cores
-// (digit.cuh) where their exactness bound allows the sides (n <= 2048), else --
-// and where the plan's memory cannot be had -- by FP64 FFTs.  One application,
-// digits against FFTs: 64 x 64 49 us / 100 us, 512 x 512 112 / 370, 1023 x 641
-// 0.24 ms / 1.79, 2048 x 2048 1.31 ms / 7.68.  Paper mode keeps the FFTs: its stop test ||P^-1 (b - M x)|| at 1e-8
+// (digit.cuh) where their exactness bound allows the sides (n <= 2048 but for 21 sides,
+// build_sine), else -- and where the plan's memory cannot be had -- by FP64 FFTs.
+// One application, digits against FFTs: 64 x 64 49 us / 100 us, 512 x 512 112 / 370, 1023 x 641
+// 0.20 ms / 1.79, 2048 x 2048 1.31 ms / 7.68.  Paper mode keeps the FFTs: its stop test ||P^-1 (b - M x)|| at 1e-8
 // is near what FP64 resolves of the penalty rows (dt/eta x cancels in b - M x),
 // so its iteration counts, which reproduce the paper's tables, depend on the rounding.
 bool left_variant(const rsfde_ctx* c) { return c->opts.variant == RSFDE_GMRES_LEFT; }

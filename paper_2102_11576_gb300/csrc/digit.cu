@@ -221,10 +221,11 @@ __global__ void __launch_bounds__(256)
 // (read once, for the largest entries and for the digits): digits dc (rows x),
 // exponents ec[x].
 //
-// The middle diagonals stay out of the digits because they are 48 to 130 times
-// the next ones: the products' absolute error is set by the largest coefficient
-// and would be 1e-15 to 5e-15 of M z (an FP64 FFT: 2e-16 to 3e-16), and is 48
-// times smaller without them; measured over 1 x 1 .. 2048 x 64, M z is then
+// The middle diagonals stay out of the digits because they are far larger than the rest: from
+// the weights of Eq. 2.6 |t0 / t2| = 12 / ((alpha - 1)(2 - alpha)), 48 at alpha = 1.5 and more
+// towards 1 and 2, and |t1 / t2| >= 22.  The products' absolute error is set by the largest
+// coefficient and would be 1e-15 to 5e-15 of M z (an FP64 FFT: 2e-16 to 3e-16); without them it is
+// at least 48 times smaller: measured over 1 x 1 .. 2048 x 64, M z is then
 // within 1.6e-16 (2-norm) of the extended-precision product, the FFTs 3.2e-16.
 template <typename Tin, int CPB>
 __global__ void __launch_bounds__(256)

@@ -13,7 +13,8 @@
 //     g_s = sum over i + j = s of sum_k d_i e_j,      s = 0..7,
 // thirty-six BF16 products into eight accumulators.  Every g_s (and every
 // partial sum of it) is an integer of at most 2^24 in magnitude -- 64 times the
-// sum of |e_j| over a row of S, which the plan checks when it builds S -- so
+// sum of |e_j| over half a row of S, which the plan checks when it builds S (21 sides
+// up to 2048 have no such digits: build_sine) -- so
 // the FP32 accumulation is exact in any order.  What is lost: the two
 // roundings to 55 bits (2^-56 of the row's largest entry; 2^-55 or 2^-56 of
 // S's) and the groups s > 7 (about 2^-54 of the result's root mean square):
