@@ -46,21 +46,21 @@ WORKLOAD = "polygon2048"
 
 # (preconditioner, operator arithmetic, Krylov basis + Gram-Schmidt, M x of the true residual)
 HEADLINE = ("bf16x3", "fp32", "fp64", "exact")
-RESID_TEXT = {"fp64": "FP64 (FFT)", "df32": "double-FP32 (FFT)",
+RESID_TEXT = {"fp64": "FP64 (FFT; digit products beside an FP64 operator)", "df32": "double-FP32 (FFT)",
               "exact": "exact (integer transforms mod four primes, Chinese remainder; rounded to FP64)"}
-PREC_TEXT = {"fp64": "FP64 (FFT)", "fp32": "FP32 (FFT)", "bf16x3": "split BF16 on tensor cores (3 products, FP32 "
+PREC_TEXT = {"fp64": "FP64 (exact digit products on tensor cores, or FFT)", "fp32": "FP32 (FFT)", "bf16x3": "split BF16 on tensor cores (3 products, FP32 "
              "accumulation)", "bf16": "plain BF16 on tensor cores (FP32 accumulation)", "df32": "double-FP32"}
 
 # ncu DRAM traffic (dram__bytes_read.sum + dram__bytes_write.sum) per unit of
 # work of a hot-path phase (one preconditioner application: its GEMM launches;
 # one Gram-Schmidt iteration: multi-dot + update), with the hash of the CUDA
 # sources that define those kernels; reported as null once any of them changes.
-# gram_schmidt: profiles/gram_schmidt_fp64_polygon2048.md, the multi-dot and
-# update of column j = 10 (FP64 basis): 813.5 MB of DRAM traffic against
+# gram_schmidt: profiles/gram_schmidt_fp64_polygon2048.md, the update of
+# column j = 9 and the multi-dot of column 10 (FP64 basis): 816.7 MB of DRAM traffic against
 # 805.3 MB of algorithmic bytes; the per-unit traffic reported is that ratio
 # times the mean algorithmic bytes of the profiled iterations.
 TRAFFIC = {
-    "gram_schmidt": {"traffic_over_algorithmic": 813473280 / 805306368, "src": "310edcbdabee4098",
+    "gram_schmidt": {"traffic_over_algorithmic": 816730368 / 805306368, "src": "4ca83ecfffa7e79c",
                      "files": ["common.cuh", "df.cuh", "internal.h", "krylov.cu"]},
 }
 
@@ -214,6 +214,16 @@ def gemm_issued_flops(n1, n2, nt):
     if n1 % 2 == 0 and n2 % 2 == 0:
         return nt * 3.0 * (n1 * n1 * n2 + n1 * n2 * n2)
     return nt * 6.0 * (n1 * n1 * n2 + n1 * n2 * n2)
+
+
+def digit_issued_flops(n1, n2, products):
+    """Tensor-core flops of `products` FP64 products of an n2 x n1 field with an axis matrix by
+    digits (half of them per axis): 36 BF16 products over both K halves, each padded to 16, for the
+    first half of the output columns.  P-hat^-1 counts six (two of its four have two channels), the
+    operator two."""
+    half = lambda n: (n + 1) // 2
+    k = lambda n: (half(n) + 15) // 16 * 32
+    return products / 2 * 36 * 2.0 * (n2 * half(n1) * k(n1) + n1 * half(n2) * k(n2))
 
 
 def max_over_ranks(value, device=None):
@@ -419,29 +429,25 @@ def run_ours(args, rank, world, local_rank):
                                    "peak_TFLOPs": pk, "frac": round(tfs / pk, 4),
                                    "peak_source": "MEASURED_PEAKS.json bf16_tflops_sustained (of measured)"}
     if plain is not None and plain["prof"]:
-        # the FP64 form's transforms are FP64-ALU bound: its flops over the FP64 peak
+        # the FP64 form's preconditioner, operator and true residual as digit products: their
+        # MMAs' flops over the phases' times (splits, folds and the residual's norm included).
+        # No row-pass launches of a phase's FFT form in the profile: it ran as digit products
         kern = plain["prof"]["kernels"]
-        L1 = 16
-        while L1 < 2 * n1 - 1:
-            L1 *= 2
-        L2 = 16
-        while L2 < 2 * n2 - 1:
-            L2 *= 2
-        pst = plain["prof"]["stats"]
-        it = sum(s["iters"] for s in pst)
-        nres = sum(s["restarts"] + 1 for s in pst) + len(pst)
-        # per application: complex FFT pair of length L per two vectors and direction,
-        # 5 L log2 L flops per transform; the operator's and the residual's rows and
-        # columns (the preconditioner runs on the tensor cores)
-        fft = lambda L: 5.0 * L * math.log2(L)
-        op_fl = (n2 / 2) * 2 * fft(L1) + (n1 / 2) * 2 * fft(L2)
-        t_op = sum(kern[k][0] for k in ("toeplitz_rows", "toeplitz_cols", "resid_rows", "resid_cols"))
-        fl = op_fl * (it + nres)
-        pk = fp64_peak_gflops(peaks.get("sm_max_mhz", 2070.0))
-        plain["fp64_roofline"] = {"transform_gflop": round(fl / 1e9, 2), "transform_ms": round(t_op, 2),
-                                  "achieved_GFLOPs": round(fl / (t_op / 1e3) / 1e9, 1),
-                                  "peak_GFLOPs": round(pk, 1), "frac": round(fl / (t_op / 1e3) / 1e9 / pk, 4),
-                                  "peak_source": "152 SMs x 2 DFMA/clk x 2 flop x sm_max_mhz (derived)"}
+        t_phase = {}
+        for k, (ms_k, _) in kern.items():
+            t_phase[PHASE_OF.get(k, "other")] = t_phase.get(PHASE_OF.get(k, "other"), 0.0) + ms_k
+        units = phase_units(plain["form"], N, plain["prof"]["stats"], m)
+        pk = peaks["bf16_tflops"]
+        plain["digit_products"] = {}
+        for ph, fft in (("precond", kern["dst_rows"][1]), ("operator", kern["toeplitz_rows"][1]),
+                        ("residual", kern["toeplitz_rows"][1])):
+            if not fft and t_phase.get(ph, 0.0) > 0:
+                fl = digit_issued_flops(n1, n2, 6 if ph == "precond" else 2)
+                us = 1e3 * t_phase[ph] / units[ph][1]
+                plain["digit_products"][ph] = {
+                    "issued_tflop_per_unit": round(fl / 1e12, 4), "us_per_unit": round(us, 2),
+                    "achieved_TFLOPs": round(fl / us / 1e6, 1), "peak_TFLOPs": pk, "frac": round(fl / us / 1e6 / pk, 4),
+                    "peak_source": "MEASURED_PEAKS.json bf16_tflops (of measured)"}
     # whole-step HBM roofline (the metric's "% HBM roofline"): the library's
     # algorithmic byte count of every step over the step time
     ach_gbs = head["bytes_per_step"] / (head["ms"] / head["steps"] / 1e3) / 1e9
@@ -527,8 +533,8 @@ def run_ours(args, rank, world, local_rank):
               "hbm_frac_step": round(f["bytes_per_step"] / (f["ms"] / f["steps"] / 1e3) / 1e9 / peaks["hbm_gbs"], 4),
               "kernels_ms": ({k: round(v[0], 2) for k, v in f["prof"]["kernels"].items() if v[1]}
                              if f["prof"] else None)}
-        if "fp64_roofline" in f:
-            fm["fp64_roofline"] = f["fp64_roofline"]
+        if f.get("digit_products"):
+            fm["digit_products"] = f["digit_products"]
         if f is not head and f["steps"] == args.steps:
             a, b = head["u"], f["u"]
             fm["headline_vs_this_rel_maxnorm_diff"] = float((a - b).abs().max() / b.abs().max())
