@@ -422,9 +422,10 @@ int ensure_bf16(rsfde_ctx* c) {
 // (digit.cuh) where their exactness bound allows the sides (n <= 2048 but for 21 sides,
 // build_sine), else -- and where the plan's memory cannot be had -- by FP64 FFTs.
 // One application, digits against FFTs: 64 x 64 49 us / 100 us, 512 x 512 112 / 370, 1023 x 641
-// 0.20 ms / 1.79, 2048 x 2048 1.31 ms / 7.68.  Paper mode keeps the FFTs: its stop test ||P^-1 (b - M x)|| at 1e-8
-// is near what FP64 resolves of the penalty rows (dt/eta x cancels in b - M x),
-// so its iteration counts, which reproduce the paper's tables, depend on the rounding.
+// 0.20 ms / 1.79, 2048 x 2048 1.28 ms / 7.68.  Paper mode keeps the FFTs: its stop test ||P^-1 (b - M x)|| at 1e-8
+// is near what FP64 resolves of the penalty rows (dt/eta x cancels in b - M x), so its
+// iteration counts, which reproduce the paper's tables, may follow the rounding (not measured
+// with digit products).
 bool left_variant(const rsfde_ctx* c) { return c->opts.variant == RSFDE_GMRES_LEFT; }
 // The FP64 operator on the Arnoldi vectors runs as digit products by the same
 // rule.  M z, digits against FFTs: 64 x 64 28 us / 56, 300 x 1500 89 / 218, 512 x
